@@ -209,31 +209,48 @@ pifepic_status pifepic_set_bedrock(pifepic_ctx* ctx, double z_bed, double eps_be
  * and 0 < margin <= 1. */
 pifepic_status pifepic_set_refinement(pifepic_ctx* ctx, double reduction, double margin);
 
-/* Preconditioner of the MIXED inner PCG of a single context (Sec. 2.5 names
- * the PCG but no preconditioner).  JACOBI: the diagonal, as the FP64 path and
+/* Preconditioner of the MIXED inner PCG (Sec. 2.5 names the PCG but no
+ * preconditioner).  JACOBI: the diagonal, as the FP64 path and
  * the oracle.  MULTIGRID: one geometric V(1,1) cycle per iteration -- coarse
  * levels at the even nodes of each axis (plus the last node of an odd axis),
  * trilinear prolongation with zero Dirichlet correction, restriction its
  * transpose, Galerkin coarse operators (27-point, built at set-up), damped
  * Jacobi smoothing (weight 0.6), the coarsest level (at most 256 nodes)
- * solved exactly by its dense inverse.  AUTO (the default): MULTIGRID for
- * meshes too large for the register-resident solver (more than 8 nodes per
- * thread of a full grid, about 620,000 nodes), where the Jacobi iteration
- * count outgrows the cap, else JACOBI -- until a warm-started solve of
- * pifepic_solve or pifepic_step (any but the context's first, which starts
- * from zero) ends at the iteration cap without converging: from then on
- * the context solves with MULTIGRID (meshes of at most 256 nodes have no
- * hierarchy and keep Jacobi).  Either solves the same system to the same
+ * solved exactly by its dense inverse.  AUTO (the default): JACOBI on a mesh
+ * that fits the register-resident solver (up to 8 nodes per thread of a full
+ * grid, about 620,000 nodes), else MULTIGRID, and where it applies in the
+ * place of either a fast-diagonalisation preconditioner: the 7-point operator
+ * with a permittivity that depends on z alone, inverted by sine or cosine
+ * transforms along x and y and tridiagonal systems along z, scaled by the
+ * node's permittivity; its iteration count does not grow with the mesh.  It
+ * applies from 32768 nodes unless every face is Neumann or an x-y plane is too
+ * large for shared memory (about 200 x 200 nodes; more than 256 along z), at
+ * once to pifepic_solve_field and in the place of MULTIGRID; in the place of
+ * JACOBI to the solves of pifepic_solve and pifepic_step after a warm-started
+ * one (any but the context's first, which starts from zero) has met the
+ * tolerance or ended a call at the iteration cap.  Its reduction is at most
+ * 1e-6 between Dirichlet faces and in a batch, else its margin at most 0.2
+ * (pifepic_set_refinement).  Where it does not apply, a warm-started Jacobi
+ * solve that ends a call at the cap without converging, like one of its own,
+ * moves the context to MULTIGRID (meshes of at most 256 nodes have no
+ * hierarchy and keep Jacobi).  All solve the same system to the same
  * stopping test.  Takes effect at once (the solve is re-planned); no
- * effect in FP64 mode or on batched solves.  Errors: EINVAL (unknown kind),
- * ENOMEM. */
+ * effect in FP64 mode.  On batched solves only AUTO has: a member whose own
+ * choice is another one is solved by Jacobi clusters.  Errors: EINVAL
+ * (unknown kind), ENOMEM. */
 enum { PIFEPIC_PRECOND_AUTO = 0, PIFEPIC_PRECOND_JACOBI = 1, PIFEPIC_PRECOND_MULTIGRID = 2 };
 pifepic_status pifepic_set_preconditioner(pifepic_ctx* ctx, int kind);
 /* The persistent solver the context's next solve runs (after AUTO's choices):
  * 1 = Jacobi PCG with the vectors in registers (meshes of at most 8 nodes per
  * thread of a full grid), 2 = Jacobi PCG with the vectors in global memory,
- * 3 = multigrid-preconditioned PCG (MIXED); 0 for a NULL context. */
-enum { PIFEPIC_SOLVER_REGISTERS = 1, PIFEPIC_SOLVER_GLOBAL = 2, PIFEPIC_SOLVER_MULTIGRID = 3 };
+ * 3 = multigrid-preconditioned PCG (MIXED), 4 = fast-diagonalisation-
+ * preconditioned PCG (MIXED); 0 for a NULL context. */
+enum {
+    PIFEPIC_SOLVER_REGISTERS = 1,
+    PIFEPIC_SOLVER_GLOBAL = 2,
+    PIFEPIC_SOLVER_MULTIGRID = 3,
+    PIFEPIC_SOLVER_FAST_DIAGONAL = 4
+};
 int pifepic_get_solver(const pifepic_ctx* ctx);
 pifepic_status pifepic_set_field_bc(pifepic_ctx* ctx, const pifepic_face_bc bc[6]);
 
@@ -399,7 +416,8 @@ pifepic_status pifepic_batch_remove(pifepic_batch* batch, pifepic_ctx* ctx);
 /* Preferred nodes per CTA of the clustered solves (a power of two from 2048
  * to 65536; 8192 is the default): a member gets the smallest cluster that
  * keeps each CTA at or under it (Jacobi clusters: also the smallest whose
- * working set fits in shared memory).  Fewer nodes per CTA is less work per
+ * working set fits in shared memory; fast-diagonalisation clusters: at or
+ * under a quarter of it).  Fewer nodes per CTA is less work per
  * iteration and more synchronisation; the serving loop's tuner picks by timing
  * steps.  EINVAL for other values. */
 pifepic_status pifepic_batch_set_cta_nodes(pifepic_batch* batch, int cta_nodes);
@@ -407,10 +425,11 @@ pifepic_status pifepic_batch_set_cta_nodes(pifepic_batch* batch, int cta_nodes);
  * member that has a multigrid hierarchy (built for the member on the first
  * step that needs it; meshes of at most 256 nodes have none and keep Jacobi)
  * by the multigrid-preconditioned PCG on one thread-block cluster of
- * ceil(nodes / cta_nodes) CTAs (1 to 16); AUTO (the default) and JACOBI keep
- * the Jacobi PCG on clusters of the member's whole working set in shared
- * memory (fewer iterations with multigrid, but each costs about eleven Jacobi
- * iterations on a cluster, and the Jacobi clusters step the batch faster).
+ * ceil(nodes / cta_nodes) CTAs (1 to 16); JACOBI solves by the Jacobi PCG on
+ * clusters of the member's whole working set in shared memory; AUTO (the
+ * default) solves the members that the fast-diagonalisation preconditioner
+ * applies to (pifepic_set_preconditioner; here from 2048 nodes) by that PCG on
+ * one cluster each, the others by Jacobi.
  * FP64 batches always use Jacobi.  The graph is rebuilt on the next step.
  * EINVAL for an unknown kind. */
 pifepic_status pifepic_batch_set_preconditioner(pifepic_batch* batch, int kind);

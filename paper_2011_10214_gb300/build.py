@@ -25,6 +25,7 @@ UNITS = [
     ("field.cu", []),
     ("pcg_coop.cu", []),
     ("pcg_mg.cu", []),
+    ("pcg_fd.cu", []),
     ("pcg_cluster.cu", []),
     ("batch.cu", []),
     ("capi.cu", ["--fmad=false"]),

@@ -19,7 +19,7 @@
 
 namespace pf {
 
-cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st);
+cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st, bool fd);
 cudaError_t launch_solve_suffix(Ctx& c, cudaStream_t st);
 int solve_graph_fixed_kernels(const Ctx& c);
 void snapshot_counters(pifepic_ctx* ctx, unsigned long long* before, long long* it0, long long* ot0, long long* l0);
@@ -30,6 +30,8 @@ pifepic_status finish_stats(pifepic_ctx* ctx, const unsigned long long* before, 
 int cluster_size_for(long long N, long long H, bool mixed, long long cta_nodes);   // pcg_cluster.cu
 cudaError_t build_pcg_graph(Ctx& c);                                                // field.cu
 cudaError_t launch_pcg_mg_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_mg.cu
+cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_fd.cu
+cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
 size_t cluster_smem_for(long long N, long long H, int C, bool mixed);
 cudaError_t launch_pcg_cluster(const BatchItem& item, int C, size_t smem, bool mixed, cudaStream_t st);
 cudaError_t launch_pcg_coop(Ctx& c, cudaStream_t st);                               // pcg_coop.cu
@@ -42,6 +44,7 @@ cudaError_t launch_movers_mixed(Ctx& c);
 cudaError_t launch_inject_mixed(Ctx& c);
 cudaError_t launch_rebin_mixed(Ctx& c);
 
+constexpr long long FD_CTA_SHARE = 4;   // fast-diagonalisation clusters: cta_nodes / 4 nodes per CTA at most
 constexpr double CL_INNER_RED = 1e-6;   // the batched Jacobi clusters' inner reduction (at most)
 
 static BatchItem make_item(Ctx& c) {
@@ -105,6 +108,21 @@ static pifepic_status batch_fail(pifepic_batch* b, pifepic_status st, const std:
 
 static long long node_halo(const Mesh& m) { return (long long)m.NX * m.NY + m.NX + 1; }
 
+// a member's cluster solves with the fast-diagonalisation preconditioner
+static bool uses_fd(const pifepic_batch* b, const Ctx& c) {
+    return b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx > 0;
+}
+
+// Its cluster: the smallest that keeps each CTA at or under a quarter of cta_nodes.  An
+// iteration is a few passes over the nodes between barriers of 0.3 us, with the
+// planes' transforms in the middle, so more CTAs pay longer than for the Jacobi
+// clusters, whose whole working set only has to fit.
+static int fd_cluster_size(long long N, long long cta_nodes) {
+    int C = 1;
+    while (C < 16 && (N + C - 1) / C > cta_nodes / FD_CTA_SHARE) C *= 2;
+    return C;
+}
+
 // The batch step as one graph: per instance a chain of its particle phases,
 // right-hand side, field solve (one cluster launch; an instance too large for
 // a cluster uses the single-instance persistent solver) and node field, so
@@ -139,6 +157,7 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             continue;
         }
         csize[i] = cluster_size_for(c.mesh.nnodes, node_halo(c.mesh), mixed, b->cta_nodes);
+        if (csize[i] > 0 && uses_fd(b, c)) csize[i] = fd_cluster_size(c.mesh.nnodes, b->cta_nodes);
     }
     const int groups[6] = {16, 8, 4, 2, 1, 0};
     std::vector<int> order;
@@ -156,12 +175,13 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
         long long l0 = c.launches;
-        e = capture(c, cs, [mixed](Ctx& cc) -> cudaError_t {
+        const bool fd = csize[i] > 0 ? uses_fd(b, c) : csize[i] == 0 && c.fd_single;
+        e = capture(c, cs, [mixed, fd](Ctx& cc) -> cudaError_t {
             cudaError_t r = mixed ? launch_push_mixed(cc) : launch_push(cc);
             if (r == cudaSuccess) r = mixed ? launch_movers_mixed(cc) : launch_movers(cc);
             if (r == cudaSuccess) r = mixed ? launch_inject_mixed(cc) : launch_inject(cc);
             if (r == cudaSuccess) r = mixed ? launch_rebin_mixed(cc) : launch_rebin(cc);
-            if (r == cudaSuccess && !cc.external_E) r = launch_solve_prefix(cc, cc.stream);
+            if (r == cudaSuccess && !cc.external_E) r = launch_solve_prefix(cc, cc.stream, fd);
             return r;
         }, &sub);
         if (e == cudaSuccess) e = cudaGraphAddChildGraphNode(&pre[i], g, nullptr, 0, sub);
@@ -182,7 +202,9 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             cudaGraph_t sub = nullptr;
             e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
-                cudaError_t e2 = launch_pcg_cluster(make_item(c), gsz, smem, mixed, cs);
+                cudaError_t e2 = uses_fd(b, c)
+                                     ? launch_pcg_fd_cluster(c, gsz, cs)
+                                     : launch_pcg_cluster(make_item(c), gsz, smem, mixed, cs);
                 e = cudaStreamEndCapture(cs, &sub);
                 if (e == cudaSuccess) e = e2;
             }
@@ -211,7 +233,9 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         if (e != cudaSuccess) break;
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
-        e = capture(c, cs, [](Ctx& cc) -> cudaError_t { return launch_pcg_coop(cc, cc.stream); }, &sub);
+        e = capture(c, cs, [](Ctx& cc) -> cudaError_t {
+            return cc.fd_single ? launch_pcg_fd(cc, cc.stream) : launch_pcg_coop(cc, cc.stream);
+        }, &sub);
         cudaGraphNode_t deps[2] = {pre[i], last_big};
         if (e == cudaSuccess) e = cudaGraphAddChildGraphNode(&solve_of[i], g, deps, last_big ? 2 : 1, sub);
         if (sub) cudaGraphDestroy(sub);

@@ -368,6 +368,16 @@ cudaError_t launch_E_to_pic(const Ctx& c, cudaStream_t st, bool both) {
     return cudaGetLastError();
 }
 
+// the solve's start vector, where its solver keeps it
+cudaError_t launch_fd_start(Ctx& c, cudaStream_t st);        // pcg_fd.cu
+cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
+static cudaError_t launch_start(Ctx& c, cudaStream_t st, bool fd) {
+    if (fd) return launch_fd_start(c, st);
+    k_u_from_phi<<<nb(c.mesh.nnodes), 256, 0, st>>>(c.mesh.nnodes, c.ntype, c.phi, c.phi_prev, c.gdir, c.u,
+                                                    solve_hist(c));
+    return cudaGetLastError();
+}
+
 static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     FieldArgs f = fargs(c);
     RhsArgs a = rargs(c);
@@ -378,10 +388,10 @@ static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     }
     k_rhs<<<node_blocks(N), node_threads(N), 0, st>>>(f, a, flux_rows(c), c.qT, c.lift, c.b, Fext,
                                                        solve_hist(c));
-    k_u_from_phi<<<nb(N), 256, 0, st>>>(N, c.ntype, c.phi, c.phi_prev, c.gdir, c.u, solve_hist(c));
-    cudaError_t e = cudaGetLastError();
+    const bool fd = Fext ? c.fd_ready : c.fd_single;
+    cudaError_t e = launch_start(c, st, fd);
     if (e != cudaSuccess) return e;
-    e = launch_pcg_coop(c, st);
+    e = fd ? launch_pcg_fd(c, st) : launch_pcg_coop(c, st);
     if (e != cudaSuccess) return e;
     if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, st);
     else k_node_E<<<node_blocks(N), node_threads(N), 0, st>>>(f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi,
@@ -391,8 +401,9 @@ static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     return launch_E_to_pic(c, st, c.precision != PIFEPIC_MIXED);
 }
 
-// the solve's pieces around the PCG, for the batched step (batch.cu)
-cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st) {
+// the solve's pieces around the PCG, for the batched step (batch.cu); fd: the
+// member's solve is the fast-diagonalisation one
+cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st, bool fd) {
     FieldArgs f = fargs(c);
     RhsArgs a = rargs(c);
     long long N = c.mesh.nnodes;
@@ -400,8 +411,7 @@ cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st) {
     if (c.nit > 0) k_qtets<<<nb(c.nit), 256, 0, st>>>(c.nit, c.it_acc, c.qcut, c.qT);
     k_rhs<<<node_blocks(N), node_threads(N), 0, st>>>(f, a, flux_rows(c), c.qT, c.lift, c.b, nullptr,
                                                        solve_hist(c));
-    k_u_from_phi<<<nb(N), 256, 0, st>>>(N, c.ntype, c.phi, c.phi_prev, c.gdir, c.u, solve_hist(c));
-    return cudaGetLastError();
+    return launch_start(c, st, fd);
 }
 cudaError_t launch_solve_suffix(Ctx& c, cudaStream_t st) {
     FieldArgs f = fargs(c);
@@ -446,6 +456,14 @@ static cudaError_t set_pcg_state(Ctx& c) {
     h.inner_red2 = c.inner_red * c.inner_red;
     h.margin2 = c.inner_margin * c.inner_margin;
     return cudaMemcpyAsync(c.scal, &h, sizeof(PcgState), cudaMemcpyHostToDevice, c.stream);
+}
+
+// whether the last solve met the tolerance (waits for the stream)
+cudaError_t last_solve_converged(Ctx& c, bool* conv) {
+    PcgState hs;
+    cudaError_t e = scopy(c.stream, &hs, pcg_state(c), sizeof(PcgState), cudaMemcpyDeviceToHost);
+    *conv = e == cudaSuccess && hs.converged;
+    return e;
 }
 
 cudaError_t launch_pcg(Ctx& c) {

@@ -33,6 +33,40 @@ struct MgLevel {                  // a coarse level (27-point Galerkin rows)
     float *b = nullptr, *x = nullptr, *res = nullptr, *y = nullptr;   // cycle vectors [N]
 };
 
+// ---- fast-diagonalisation preconditioner of the MIXED field solve (pcg_fd.cu) ----
+// AUTO uses it from this many nodes: below, a Jacobi iteration (3 us) is cheap enough that
+// its 60 or so beat 14 of these at 17 us (24^3 sphere: 0.23 against 0.26 ms a solve; 32^3:
+// 0.27 against 0.23, 37^3 0.34 against 0.31, 64^3 0.70 against 0.32)
+constexpr long long FD_MIN_NODES = 32768;
+// a batch's clusters from this many (16^3 cells: 0.26 ms a member's step against 0.45 with
+// the Jacobi cluster, 48^3: 0.66 against 1.52)
+constexpr long long FD_CLUSTER_MIN_NODES = 2048;
+struct FdPlan {
+    int mx = 0, my = 0, mz = 0;   // free nodes per axis (0: no plan), the first at (x0, y0, z0)
+    int x0 = 0, y0 = 0, z0 = 0;
+    bool deep = false;            // inner solves reduce the residual 1e-6-fold (every face Dirichlet)
+    int ksx = 0, ksy = 0;         // 16-node steps along x and y
+    int ldX = 0, ldY = 0, ldT = 0;   // row strides: plane and first product in shared memory (pairs), modes
+    int nch = 0, mta = 0;         // column chunks of a plane, their 16-column tiles
+    int pb = 1;                   // planes a block transforms at a time
+    int nt1 = 0, nt2 = 0;         // 8-column tiles a warp takes at a time, per product
+    int stage = 0;                // where the fragments start in shared memory (pairs; 0: read from global memory)
+    int ldv = 0, PV = 0;          // the box of the vectors: row and plane strides
+    long long PT = 0;             // modes of a plane (padded)
+    double* u = nullptr;          // the unknown (FP64), inside a zeroed guard; [mz][PV], as the vectors below
+    float* z = nullptr;           // inside a zeroed guard
+    float *r[2] = {nullptr, nullptr}, *q[2] = {nullptr, nullptr};   // two copies: one read, one written
+    float *w = nullptr, *p = nullptr, *x = nullptr;
+    const float* s = nullptr;     // diagonal scaling
+    const unsigned char* kind = nullptr;   // node kinds
+    const int* patch = nullptr;   // [npatch] the patch rows' places
+    float* T = nullptr;           // [mz][PT] transformed residual
+    const float* inv = nullptr;   // [mz][PT] inverted pivots
+    const float* ez = nullptr;    // [mz] couplings along z
+    const uint4 *fxF = nullptr, *fxI = nullptr;   // split basis matrices in fragment order: to modes, back
+    const uint4 *fyF = nullptr, *fyI = nullptr;
+};
+
 // ---- particle arrays (SoA) -------------------------------------------------
 struct PArr {            // FP64 mode: xi in cell units, physical velocity
     double *x, *y, *z, *vx, *vy, *vz;
@@ -240,7 +274,13 @@ struct Ctx {
     float* mg_r0 = nullptr;           // fine residual after pre-smoothing
     float* mg_cinv = nullptr;         // dense inverse of the coarsest operator
     bool mg_wanted = false;           // a batch solves this context with multigrid: keep a hierarchy
-    bool mg_escalated = false;        // AUTO: a Jacobi solve ended at the cap unconverged; multigrid since
+    bool mg_escalated = false;        // AUTO: a Jacobi solve ended at the cap unconverged; another solver since
+    bool fd_capped = false;           // AUTO: a fast-diagonalisation solve did; multigrid since
+    FdPlan fd;                        // fast-diagonalisation preconditioner (fd.mx = 0: none)
+    bool fd_ready = false;            // pifepic_solve_field uses it
+    bool fd_now = false;              // a warm-started Jacobi solve is done: the steps use it too
+    bool fd_single = false;           // the solves of pifepic_solve and pifepic_step use it
+    char* fd_mem = nullptr;           // its arrays
     long long solves_done = 0;        // field solves of pifepic_solve and pifepic_step so far
     cudaStream_t side = nullptr;      // movers and injection beside the push (pifepic_step)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

@@ -725,6 +725,7 @@ static void plan_pcg_reg(Ctx& c);
 // the register-resident plan, else the global-memory kernel's row kinds and
 // FP64 correction vector (made here, before any capture of the solve)
 cudaError_t plan_pcg_mg(Ctx& c);   // pcg_mg.cu: the multigrid hierarchy (MIXED), if selected
+cudaError_t plan_pcg_fd(Ctx& c);   // pcg_fd.cu: the fast-diagonalisation preconditioner (MIXED), if selected
 
 void plan_pcg(Ctx& c) {
     // the exchanges count arrivals in multiples of their grid size, which differs
@@ -735,8 +736,9 @@ void plan_pcg(Ctx& c) {
     plan_pcg_reg(c);
     lib_free(c.rowkind); lib_free(c.pcg_x);
     c.rowkind = nullptr; c.pcg_x = nullptr;
+    if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();   // (no plan: the solvers below)
     if (plan_pcg_mg(c) != cudaSuccess) cudaGetLastError();   // (no hierarchy: the Jacobi solvers)
-    if (c.pcg_npt > 0 && c.mg_nlev == 0) return;
+    if ((c.pcg_npt > 0 || c.fd_single) && c.mg_nlev == 0) return;
     const long long N = c.mesh.nnodes;
     if (lib_malloc(&c.rowkind, sizeof(unsigned short) * N) != cudaSuccess ||
         lib_malloc(&c.pcg_x, sizeof(double) * N) != cudaSuccess) {

@@ -30,13 +30,9 @@
 #include <cstring>
 #include <vector>
 
-#include <cooperative_groups.h>
-
 #include "field_common.cuh"
 #include "internal.h"
-#include "pcg_sync.cuh"
-
-namespace cg = cooperative_groups;
+#include "pcg_team.cuh"
 
 namespace pf {
 
@@ -175,21 +171,6 @@ static __device__ __forceinline__ void fine_ijk(const Mesh& m, long long n, int&
     k = (int)(t / (unsigned)m.NY);
 }
 
-// a fine row times v (v inside a zeroed guard: the masked stencil reads the
-// absent neighbours of boundary nodes and multiplies them by zero)
-static __device__ __forceinline__ float mg_fine_row(const FieldArgs& f, const float* v, long long n, unsigned kd) {
-    if (kd & RK_DIRICHLET) return 0.0f;
-    if (kd & RK_GENERAL) {
-        int i, j, k;
-        node_ijk(f.m, n, i, j, k);
-        return apply_row<float, true>(f, n, i, j, k, v, f.coeff);
-    }
-    const int NX = f.m.NX, NXY = f.m.NX * f.m.NY;
-    return regular_row_masked_ld<float>([&](int o) { return __ldcg(v + n + o); }, NX, NXY, kd, (float)f.m.h,
-                                        h_over6<float>(f.m), h_over12<float>(f.m), (float)f.o.eps_plus,
-                                        (float)f.o.eps_minus);
-}
-
 // ---- Galerkin coarse operators (set-up) ------------------------------------------------
 // the 19 slots of a fine row (row_coeffs order)
 __constant__ int cSlot19[19][3] = {{0, 0, 0},  {-1, 0, 0}, {1, 0, 0},  {0, -1, 0}, {0, 1, 0},  {0, 0, -1}, {0, 0, 1},
@@ -290,93 +271,7 @@ __global__ void k_mg_rap(MgLevel F, MgLevel C) {
     rap_store(C, I, acc);
 }
 
-// ---- the team that solves one system ---------------------------------------------------
-// GridTeam: the whole cooperative grid (one system per launch; grid barriers and
-// exchanges over the arrival counter, bounded waits).  ClusterTeam: one
-// thread-block cluster per system (a batch of independent systems per launch;
-// the hardware cluster barrier orders global memory within the cluster, and a
-// reduction reads the C block partials through distributed shared memory).
-struct GridTeam {
-    const MgArgs& a;
-    int& e;
-    ExchShared& xs;
-    __device__ long long t0() const { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
-    __device__ long long size() const { return (long long)gridDim.x * blockDim.x; }
-    __device__ bool leader() const { return blockIdx.x == 0; }
-    __device__ bool sync() { return grid_barrier(a, e, xs); }
-    template <typename A, int NV>
-    __device__ bool reduce(A (&v)[NV], A (&tot)[NV]) { return exchange<A, NV>(a, e, v, tot, xs); }
-};
-
-struct ClusterSlots {
-    double sh[4 * 32];
-    double bc[4];
-    double slot[2][4];    // this CTA's partials, by reduction parity
-};
-
-struct ClusterTeam {
-    cg::cluster_group& cl;
-    int C, rank;
-    int e;
-    ClusterSlots& cs;
-    __device__ long long t0() const { return (long long)rank * blockDim.x + threadIdx.x; }
-    __device__ long long size() const { return (long long)C * blockDim.x; }
-    __device__ bool leader() const { return rank == 0; }
-    __device__ bool sync() {
-        cl.sync();
-        return true;
-    }
-    // every CTA of the cluster gets the same totals (the partials summed in rank order)
-    template <typename A, int NV>
-    __device__ bool reduce(A (&v)[NV], A (&tot)[NV]) {
-        A* sh = (A*)cs.sh;
-        block_sum_t<A, NV>(v, sh);
-        A* slot = (A*)cs.slot[e & 1];
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int q = 0; q < NV; ++q) slot[q] = v[q];
-        cl.sync();
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-#pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                A x = (A)0;
-                if (lane < C) x = cl.map_shared_rank(slot, lane)[q];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-                if (lane == 0) ((A*)cs.bc)[q] = x;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < NV; ++q) tot[q] = ((A*)cs.bc)[q];
-        ++e;
-        return true;
-    }
-};
-
 // ---- the V-cycle ---------------------------------------------------------------------
-// A pass over the nodes [0, N) of a level, strided over the grid, four nodes
-// at a time: every node's value (its loads) before any node's store, so the
-// L2 round trips of a group overlap.
-constexpr int MG_UNROLL = 4;
-template <class F, class S>
-static __device__ __forceinline__ void pass4(long long N, long long t0, long long TT, F value, S store) {
-    for (long long n0 = t0; n0 < N; n0 += MG_UNROLL * TT) {
-        float v[MG_UNROLL];
-#pragma unroll
-        for (int u = 0; u < MG_UNROLL; ++u) {
-            const long long n = n0 + u * TT;
-            v[u] = n < N ? value(n) : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < MG_UNROLL; ++u) {
-            const long long n = n0 + u * TT;
-            if (n < N) store(n, v[u]);
-        }
-    }
-}
-
 // the pre-smoothing step from a zero start, x0 = omega D^-1 r: no product, so
 // the passes that produce r write it node by node
 static __device__ __forceinline__ float mg_presmooth(const FieldArgs& f, long long n, float rn) {
@@ -395,7 +290,7 @@ static __device__ bool vcycle(const MgArgs& a, Team& team, float* sb, float (&rz
     const Dims d0 = dims_of(f.m);
     // level 0, down: the residual after pre-smoothing
     if (!team.sync()) return false;
-    pass4(N, t0, TT, [&](long long n) { return __ldcg(a.r + n) - mg_fine_row(f, a.x0, n, a.kind[n]); },
+    pass4(N, t0, TT, [&](long long n) { return __ldcg(a.r + n) - fine_row_f(f, a.x0, n, a.kind[n]); },
           [&](long long n, float v) { a.r0[n] = v; });
     if (!team.sync()) return false;
     // coarse levels above the coarsest, down: restriction and pre-smoothing, then the residual
@@ -498,21 +393,21 @@ static __device__ bool vcycle(const MgArgs& a, Team& team, float* sb, float (&rz
     if (!team.sync()) return false;
     rz[0] = 0.0f;
     rz[1] = 0.0f;
-    for (long long n0 = t0; n0 < N; n0 += MG_UNROLL * TT) {
-        float zv[MG_UNROLL], rv[MG_UNROLL];
+    for (long long n0 = t0; n0 < N; n0 += PASS_UNROLL * TT) {
+        float zv[PASS_UNROLL], rv[PASS_UNROLL];
 #pragma unroll
-        for (int u = 0; u < MG_UNROLL; ++u) {
+        for (int u = 0; u < PASS_UNROLL; ++u) {
             const long long n = n0 + u * TT;
             zv[u] = 0.0f;
             rv[u] = 0.0f;
             if (n < N) {
                 const float xn = __ldcg(a.x0 + n);
                 rv[u] = __ldcg(a.r + n);
-                zv[u] = xn + MG_OMEGA * f.invdiagf[n] * (rv[u] - mg_fine_row(f, a.x0, n, a.kind[n]));
+                zv[u] = xn + MG_OMEGA * f.invdiagf[n] * (rv[u] - fine_row_f(f, a.x0, n, a.kind[n]));
             }
         }
 #pragma unroll
-        for (int u = 0; u < MG_UNROLL; ++u) {
+        for (int u = 0; u < PASS_UNROLL; ++u) {
             const long long n = n0 + u * TT;
             if (n < N) a.z[n] = zv[u];
             rz[0] += rv[u] * zv[u];
@@ -578,7 +473,7 @@ static __device__ void mg_pcg(const MgArgs& a, Team& team, float* sb) {
             rz = t2[0];
             // p = z + beta p, q = A z + beta q (= A p)
             float v1[1] = {0.0f};
-            pass4(N, t0, TT, [&](long long n) { return mg_fine_row(f, z, n, a.kind[n]); },
+            pass4(N, t0, TT, [&](long long n) { return fine_row_f(f, z, n, a.kind[n]); },
                   [&](long long n, float az) {
                       const float zn = __ldcg(z + n);
                       const float pn = first ? zn : zn + beta * p[n];
@@ -620,7 +515,7 @@ __global__ void __launch_bounds__(MG_THREADS, 1) k_pcg_mg(MgArgs a) {
     __shared__ ExchShared xs;
     __shared__ float sb[MG_COARSEST];   // the coarsest right-hand side (block 0)
     int e = 0;
-    GridTeam team{a, e, xs};
+    GridTeam<MgArgs> team{a, e, xs};
     mg_pcg(a, team, sb);
 }
 
@@ -715,7 +610,7 @@ cudaError_t plan_pcg_mg(Ctx& c) {
     // cap; and once a Jacobi solve of this context has ended at the cap
     // unconverged (mostly Neumann faces: poorly conditioned for Jacobi)
     const bool single = c.precond == PIFEPIC_PRECOND_MULTIGRID ||
-                        (c.precond == PIFEPIC_PRECOND_AUTO && (c.pcg_npt == 0 || c.mg_escalated));
+                        (c.precond == PIFEPIC_PRECOND_AUTO && !c.fd_single && (c.pcg_npt == 0 || c.mg_escalated));
     if (!single && !c.mg_wanted) return cudaSuccess;
     const long long N0 = c.mesh.nnodes;
     int nx = c.mesh.nx, ny = c.mesh.ny, nz = c.mesh.nz;

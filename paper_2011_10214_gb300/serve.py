@@ -252,8 +252,8 @@ class Server:
 
 
 def autotune_batch(batch, trial_steps=2, candidates=(8192, 4096, 2048),
-                   preconds=(capi.PRECOND_MULTIGRID, capi.PRECOND_JACOBI)):
-    """Pick the clustered solves' preconditioner (multigrid or Jacobi) and
+                   preconds=(capi.PRECOND_AUTO, capi.PRECOND_MULTIGRID, capi.PRECOND_JACOBI)):
+    """Pick the clustered solves' preconditioner (automatic, multigrid or Jacobi) and
     nodes per CTA (hence each member's cluster size) by timing real steps of
     the batch (the trial steps advance the members like any other step).
     Returns (preconditioner, nodes per CTA, seconds per step of the pick)."""

@@ -1,0 +1,136 @@
+"""The fast-diagonalisation PCG (pcg_fd.cu) against the oracle's solve, at shapes
+where its tiles, runs and padding have their edges.
+
+Both sides iterate to ||r|| <= 1e-12 ||b|| on the same system, so the potentials
+agree to about cond(A) * 1e-12; the bar is 1e-8 relative (max norm), as for the
+other solvers."""
+import numpy as np
+import pytest
+
+from oracle.geometry import Mesh
+from oracle.pic import Simulation as OracleSim
+from tests.pairs import add_species_both, explicit_particles, gpu_object, oracle_object
+
+pytestmark = pytest.mark.gpu
+
+TOL_PHI = 1e-8
+D, N = ("D", 0.2), ("N",)
+
+
+def _pair(n, bc, obj, bed=None, maxit=5000, tol=1e-12):
+    from paper_2011_10214_gb300 import capi
+    m = Mesh(*n, 0.5)
+    orc = OracleSim(m, oracle_object(m, obj, bed), bc, 0.05, tol=1e-12, maxit=5000)
+    gpu = capi.Simulation(n, 0.5, 0.05, precision=capi.MIXED, pcg_tol=tol, pcg_max_iter=maxit, track_ids=True)
+    gpu.set_field_bc(bc)
+    gpu_object(gpu, obj, bed)
+    return gpu, orc
+
+
+def _sphere(n, eps=6.0):
+    return ("sphere", tuple(0.25 * v for v in n), 0.11 * min(n), eps, 1.0)
+
+
+# (cells, faces, object, bedrock): free nodes per axis at and around the 16-node tiles, z runs of 8 rows on 8 and 16
+# warps, planes in column chunks
+SINGLE = [
+    ((33, 32, 31), [D] * 6, None, None),                            # 32 x 31 x 30 free nodes
+    ((32, 33, 34), [N, D, D, N, N, D], None, None),                 # 32 x 33 x 34
+    ((17, 19, 100), [D, D, N, D, D, D], None, None),                # 16 x 19 x 99
+    ((100, 100, 5), [D] * 6, ("none",), None),                      # 99 x 99 x 4: planes in column chunks
+]
+# an axis Neumann at both ends, objects on the faces, layers: Jacobi until a solve is capped
+OPEN = [
+    ((40, 36, 24), [N] * 5 + [D], ("cap_crater", 4.1, 10.0, 9.0, 6.0, 2.0, 4.0, 1.0), None),
+    ((48, 24, 30), [N] * 5 + [D], ("rim_crater", 4.87, 12.0, 0.0, 2.1, 3.9, 5.6, 1.3, 1.1, 4.0, 1.0), (2.4, 10.0)),
+]
+
+
+@pytest.mark.parametrize("case", range(len(SINGLE)))
+def test_fast_diagonal_solve_matches_oracle(case):
+    from paper_2011_10214_gb300 import capi
+    n, bc, obj, bed = SINGLE[case]
+    gpu, orc = _pair(n, bc, obj or _sphere(n), bed)
+    fs = orc.fs
+    g = np.random.default_rng(100 + case)
+    for _ in range(2):                       # the second starts from the first's potential
+        F = g.normal(size=fs.mesh.nnodes) * fs.mesh.h ** 3
+        q = g.normal(size=len(fs.it_cell))
+        phi, _, _ = fs.solve(F, q, tol=1e-12, maxit=5000)
+        _, rr = gpu.solve_field(F, q)
+        assert rr <= 1e-12
+        assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max()
+    gpu.close()
+
+
+@pytest.mark.parametrize("case", range(len(OPEN)))
+def test_capped_jacobi_solves_move_to_fast_diagonal(case):
+    from paper_2011_10214_gb300 import capi
+    n, bc, obj, bed = OPEN[case]
+    gpu, orc = _pair(n, bc, obj, bed, maxit=80)
+    add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+    explicit_particles(gpu, orc, 0, 4000, 5, 1.0)
+    for _ in range(2):                       # the second, warm-started, moves the context on
+        assert gpu.solver == capi.SOLVER_REGISTERS
+        st = gpu.solve()
+        assert st["pcg_converged"] == 0 and st["pcg_iters"] == 80
+    assert gpu.solver == capi.SOLVER_FAST_DIAGONAL
+    st = gpu.solve()
+    assert st["pcg_converged"] == 1 and st["pcg_iters"] < 80
+    orc.solve()
+    assert np.abs(gpu.potential() - orc.phi).max() <= TOL_PHI * np.abs(orc.phi).max()
+    gpu.close()
+
+
+@pytest.mark.parametrize("steps", [1, 6])
+def test_steps_move_to_fast_diagonal_after_a_warm_solve(steps):
+    """The cold first solve and a warm one run Jacobi; the context moves on at the
+    end of the call, or at its fifth step.  P is singular without a Dirichlet face
+    (and so is the system: its capped solve leads to multigrid), small meshes keep
+    Jacobi, an explicit choice stands."""
+    from paper_2011_10214_gb300 import capi
+    R, F, G = capi.SOLVER_REGISTERS, capi.SOLVER_FAST_DIAGONAL, capi.SOLVER_MULTIGRID
+    for n, bc, pc, before, after in (((32, 32, 32), [D] * 6, None, R, F), ((32, 32, 32), [N] * 6, None, R, G),
+                                     ((24, 24, 24), [D] * 6, None, R, R),
+                                     ((32, 32, 32), [D] * 6, capi.PRECOND_JACOBI, R, R),
+                                     ((32, 32, 32), [D] * 6, capi.PRECOND_MULTIGRID, G, G)):
+        gpu, orc = _pair(n, bc, _sphere(n), maxit=1000, tol=1e-6)
+        if pc is not None:
+            gpu.set_preconditioner(pc)
+        add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+        explicit_particles(gpu, orc, 0, 4000, 5, 1.0)
+        gpu.solve()
+        assert gpu.solver == before
+        st = gpu.step(steps)
+        assert gpu.solver == after, (n, bc, pc)
+        if after == F:
+            assert st["pcg_converged"] == 1 and (steps == 1 or st["pcg_iters"] < 25)
+        gpu.close()
+
+
+# members of a batch: clusters of 2 to 16 CTAs, a CTA's planes transformed in groups; every pair of ends, one free
+# node along an axis, z runs of 16 rows
+BATCH = [((13, 12, 14), [D] * 6), ((17, 16, 15), [N, D, D, D, N, D]), ((24, 33, 9), [D, D, N, N, D, N]),
+         ((31, 18, 47), [D, N, N, D, D, D]), ((48, 46, 49), [D] * 6), ((2, 33, 30), [D, D, N, N, D, N]),
+         ((40, 2, 30), [N, D, D, D, N, N]), ((33, 40, 2), [N, N, N, N, D, D]), ((8, 8, 140), [N, D, D, N, D, D])]
+
+
+def test_fast_diagonal_clusters_match_oracle():
+    from paper_2011_10214_gb300 import capi
+    pairs = [_pair(n, bc, _sphere(n) if min(n) > 2 else ("none",)) for n, bc in BATCH]
+    for k, (gpu, orc) in enumerate(pairs):
+        add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+        explicit_particles(gpu, orc, 0, 3000, 50 + k, 0.5)
+    batch = capi.Batch([gpu for gpu, _ in pairs])
+    for _ in range(2):
+        st = batch.step(1)
+        for k, (gpu, orc) in enumerate(pairs):
+            assert st[k]["pcg_converged"] == 1 and st[k]["pcg_relres"] <= 1e-12
+            # the oracle's solution for the charges that the member deposited
+            F = gpu.node_charge(0) * (-0.01 / 2.0 ** 32)
+            qT = orc.fs.q_tets(-0.01 * gpu.surface_counts(0).astype(np.float64))
+            phi, _, _ = orc.fs.solve(F, qT, tol=1e-12, maxit=5000)
+            assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max(), BATCH[k]
+    batch.close()
+    for gpu, _ in pairs:
+        gpu.close()
