@@ -628,11 +628,7 @@ static pifepic_status ensure_movers(pifepic_ctx* ctx, int s, long long need) {
         if (e == cudaSuccess) e = alloc_parrf(f1, need, c.track != 0);
         if (e != cudaSuccess) FAIL(PIFEPIC_ENOMEM, "mover list allocation failed");
         if (keep > 0) {
-            CUDA_OK(scopy(c.stream, f0.cell, q.movF[0].cell, sizeof(int) * keep, cudaMemcpyDeviceToDevice));
-            float* src[6] = {q.movF[0].fx, q.movF[0].fy, q.movF[0].fz, q.movF[0].vx, q.movF[0].vy, q.movF[0].vz};
-            float* dst[6] = {f0.fx, f0.fy, f0.fz, f0.vx, f0.vy, f0.vz};
-            for (int d = 0; d < 6; ++d)
-                CUDA_OK(scopy(c.stream, dst[d], src[d], sizeof(float) * keep, cudaMemcpyDeviceToDevice));
+            CUDA_OK(scopy(c.stream, f0.w, q.movF[0].w, sizeof(unsigned) * PGROUP * ((keep + 31) / 32), cudaMemcpyDeviceToDevice));
             if (c.track) CUDA_OK(scopy(c.stream, f0.id, q.movF[0].id, sizeof(long long) * keep, cudaMemcpyDeviceToDevice));
         }
         PArrF old0 = q.movF[0], old1 = q.movF[1];
@@ -1060,12 +1056,7 @@ static pifepic_status fill_stats(pifepic_ctx* ctx, const unsigned long long* bef
     if (herr & ERR_TMA_TIMEOUT) {
         szero(c.stream, c.err_word, sizeof(int));
         cudaStreamSynchronize(c.stream);
-        FAIL(PIFEPIC_ETIMEOUT, "a node-field tile load timed out");
-    }
-    if (herr & ERR_CHUNK_TIMEOUT) {
-        szero(c.stream, c.err_word, sizeof(int));
-        cudaStreamSynchronize(c.stream);
-        FAIL(PIFEPIC_ETIMEOUT, "a bin's compaction order wait timed out (its particles were dropped)");
+        FAIL(PIFEPIC_ETIMEOUT, "a node-field tile or particle load timed out (the bin's particles may have been dropped)");
     }
     if (herr & ERR_BARRIER_TIMEOUT) {
         // the barrier counters are left mid-count: clear them and the flag so

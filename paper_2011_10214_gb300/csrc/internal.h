@@ -73,12 +73,18 @@ struct PArr {            // FP64 mode: xi in cell units, physical velocity
     long long* id;
     void* base;          // the one allocation holding all arrays (null: allocated one by one)
 };
-struct PArrF {           // MIXED mode: packed cell (i | j<<11 | k<<22), FP32 offset and velocity
-    int* cell;
-    float *fx, *fy, *fz, *vx, *vy, *vz;
+// MIXED mode: a packed cell (i | j<<11 | k<<22), FP32 offset in the cell and velocity, in
+// groups of 32 particles: the 32 cells, then the 32 x offsets, y, z, vx, vy, vz.  A warp's
+// particles are one run of 896 bytes: one bulk copy in, one address and fixed distances
+// for the seven words out
+constexpr int PGROUP = 7 * 32;       // words of a group
+struct PArrF {
+    unsigned* w;
     long long* id;
     void* base;          // as PArr::base
 };
+// the place of particle g's first word (the others 32 words apart)
+PF_HD long long pword(long long g) { return (g >> 5) * PGROUP + (g & 31); }
 
 // per-species parameters and pointers handed to kernels by value
 struct SpeciesDev {

@@ -470,7 +470,8 @@ __global__ void k_bin_caps(int nb, const int* cnt, int* cap, int* cnt_copy) {
     cnt_copy[b] = 0;
 }
 
-// exclusive scan of the bin capacities, one block of BIN_SCAN_THREADS: each
+// exclusive scan of the bin capacities rounded up to 32 slots (a bin starts on a
+// 128-byte boundary of every array), one block of BIN_SCAN_THREADS: each
 // thread sums a contiguous run of bins, the runs' totals are scanned across
 // the block, then each thread writes its run's starts
 __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* total) {
@@ -479,7 +480,7 @@ __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* 
     const int per = (nb + BIN_SCAN_THREADS - 1) / BIN_SCAN_THREADS;
     const int b0 = t * per, b1 = min(b0 + per, nb);
     long long mine = 0;
-    for (int b = b0; b < b1; ++b) mine += cap[b];
+    for (int b = b0; b < b1; ++b) mine += (cap[b] + 31) & ~31;
     long long inc = mine;   // inclusive scan within the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -499,7 +500,7 @@ __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* 
     }
     __syncthreads();
     long long run = inc - mine + (w > 0 ? wsum[w - 1] : 0);
-    for (int b = b0; b < b1; ++b) { start[b] = run; run += cap[b]; }
+    for (int b = b0; b < b1; ++b) { start[b] = run; run += (cap[b] + 31) & ~31; }
     if (t == BIN_SCAN_THREADS - 1) *total = wsum[BIN_SCAN_THREADS / 32 - 1];
 }
 

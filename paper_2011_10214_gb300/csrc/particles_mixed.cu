@@ -223,25 +223,21 @@ PF_D void global_deposit_f(const Launch& L, unsigned long long* W, const PF32& p
                   (unsigned long long)Wf[l]);
 }
 
-// asynchronous 4-byte global -> shared copies (cp.async), committed in groups
-PF_D void cp_async4(void* dst, const void* src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
-PF_D void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-PF_D void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-PF_D void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 PF_D void load_p(const PArrF& a, long long g, PF32& p) {
-    unpack_cell(a.cell[g], p.i, p.j, p.k);
-    p.fx = a.fx[g]; p.fy = a.fy[g]; p.fz = a.fz[g];
-    p.vx = a.vx[g]; p.vy = a.vy[g]; p.vz = a.vz[g];
+    const unsigned* w = a.w + pword(g);
+    unpack_cell((int)w[0], p.i, p.j, p.k);
+    p.fx = __uint_as_float(w[32]); p.fy = __uint_as_float(w[64]); p.fz = __uint_as_float(w[96]);
+    p.vx = __uint_as_float(w[128]); p.vy = __uint_as_float(w[160]); p.vz = __uint_as_float(w[192]);
+}
+PF_D void store_v(const PArrF& a, long long g, float vx, float vy, float vz) {
+    unsigned* w = a.w + pword(g);
+    w[128] = __float_as_uint(vx); w[160] = __float_as_uint(vy); w[192] = __float_as_uint(vz);
 }
 PF_D void store_p(const PArrF& a, long long g, const PF32& p, long long id, bool track) {
-    a.cell[g] = pack_cell(p.i, p.j, p.k);
-    a.fx[g] = p.fx; a.fy[g] = p.fy; a.fz[g] = p.fz;
-    a.vx[g] = p.vx; a.vy[g] = p.vy; a.vz[g] = p.vz;
+    unsigned* w = a.w + pword(g);
+    w[0] = (unsigned)pack_cell(p.i, p.j, p.k);
+    w[32] = __float_as_uint(p.fx); w[64] = __float_as_uint(p.fy); w[96] = __float_as_uint(p.fz);
+    w[128] = __float_as_uint(p.vx); w[160] = __float_as_uint(p.vy); w[192] = __float_as_uint(p.vz);
     if (track) a.id[g] = id;
 }
 
@@ -264,16 +260,20 @@ PF_D int block_of(const Launch& L, int ci, int cj, int ck) {
 // fused gather + push + boundary + collection + deposit + compaction (one bin per CTA)
 // ------------------------------------------------------------------------------------
 // A bin of B^3 cells reads and deposits through a TL^3 node tile, TL = B + 1.
-// gather from the staged node-field tile; t0 = tile index of the cell's corner 0
+// The node-field tile holds each node with its neighbour along x, P = (Ex, Ex', Ey, Ey') and
+// Q = (Ez, Ez'): a cell's field is 4 x (16 + 8) bytes, 24 shared-memory wavefronts a warp at
+// least, against 32 for eight float4 nodes.  t0 = tile index of the cell's corner 0; the sums
+// run over the corners in their order, as gather_f's.
 template <int TL>
-PF_D void gather_tile(const float4* Et, int t0, const WF& w, float& ex, float& ey, float& ez) {
+PF_D void gather_tile(const float4* P, const float2* Q, int t0, const WF& w, float& ex, float& ey, float& ez) {
     ex = 0.f; ey = 0.f; ez = 0.f;
 #pragma unroll
-    for (int l = 0; l < 8; ++l) {
-        const float4 e = Et[t0 + tile_corner<TL>(l)];
-        ex += w.w[l] * e.x;
-        ey += w.w[l] * e.y;
-        ez += w.w[l] * e.z;
+    for (int l = 0; l < 8; l += 2) {
+        const float4 p = P[t0 + tile_corner<TL>(l)];
+        const float2 q = Q[t0 + tile_corner<TL>(l)];
+        ex += w.w[l] * p.x; ex += w.w[l + 1] * p.y;
+        ey += w.w[l] * p.z; ey += w.w[l + 1] * p.w;
+        ez += w.w[l] * q.x; ez += w.w[l + 1] * q.y;
     }
 }
 
@@ -282,27 +282,31 @@ PF_D int tile_index(int i, int j, int k, int x0, int y0, int z0) {
     return (i - x0) + TL * ((j - y0) + TL * (k - z0));
 }
 
-// a bin's deposit tile: 8 interleaved 32-bit copies per node (copy = lane & 7),
+// a bin's deposit tile: NC interleaved 32-bit copies per node (copy = lane % NC),
 // units of 2^-19 particle (see k_push_bins_m).  One particle: 7 rounded
-// weights and the remainder, so it adds exactly 2^19.
-template <int TL>
-PF_D void tile_deposit19(unsigned* Wt, int t0, const WF& w) {
+// weights and the remainder, so it adds exactly 2^19.  (The scale, a power of
+// two, goes into the z weights: the products round the same.)
+template <int TL, int NC>
+PF_D void tile_deposit19(unsigned* Wt, int t0, float fx, float fy, float fz) {
+    const float wx[2] = {1.0f - fx, fx}, wy[2] = {1.0f - fy, fy}, wz[2] = {(1.0f - fz) * 524288.0f, fz * 524288.0f};
     unsigned rest = 1u << 19;
 #pragma unroll
     for (int l = 0; l < 7; ++l) {
-        const unsigned W = __float2uint_rn(w.w[l] * 524288.0f);
+        const unsigned W = __float2uint_rn((wx[l & 1] * wy[(l >> 1) & 1]) * wz[(l >> 2) & 1]);
         rest -= W;
-        atomicAdd(&Wt[t0 + 8 * tile_corner<TL>(l)], W);
+        atomicAdd(&Wt[t0 + NC * tile_corner<TL>(l)], W);
     }
-    atomicAdd(&Wt[t0 + 8 * tile_corner<TL>(7)], rest);
+    atomicAdd(&Wt[t0 + NC * tile_corner<TL>(7)], rest);
 }
 // add the tile to the node charges (2^32 units per particle), all threads of the block
-template <int TL>
+// (a node's copies are read from a different one on by each lane: NC = 32 would put every
+// lane's first copy into one bank)
+template <int TL, int NC>
 PF_D void tile_flush19(const Launch& L, unsigned long long* W, const unsigned* Wt, int x0, int y0, int z0) {
     for (int t = threadIdx.x; t < TL * TL * TL; t += blockDim.x) {
         long long v = 0;
-        for (int c = 0; c < 8; ++c) {
-            long long u = (long long)Wt[t * 8 + c];
+        for (int c = 0; c < NC; ++c) {
+            long long u = (long long)Wt[t * NC + ((c + t) & (NC - 1))];
             if (u >= (3ll << 30)) u -= 1ll << 32;     // a (small) negative copy total
             v += u;
         }
@@ -314,60 +318,142 @@ PF_D void tile_flush19(const Launch& L, unsigned long long* W, const unsigned* W
     }
 }
 
-// One CTA per (bin, species); warps take chunks of 32 particles in turn
-// (chunk c to warp c mod 8, prefetching the next) and never wait at a block
-// barrier.  Stayers are compacted in place: chunk c writes its stayers right
-// after those of chunks 0..c-1.  Each chunk publishes its own stayer count in
-// shared memory as soon as it has it; the warp of chunk c adds the counts of
-// chunks c-7..c-1 (one per lane: the other warps' latest chunks) to its own
-// running total up to chunk c-8, so no warp waits on a chain of publications.
-// Writes land only on slots of chunks <= c, all of which were read before
-// their counts were published, so no unread particle is overwritten.
-// A warp's next PUSH_DEPTH chunks are in flight at any time: each lane copies
-// its particle's seven words into the warp's stage in shared memory with
-// cp.async (no registers held while the loads travel) and reads them back
-// when the chunk comes up.
+// One CTA of NW warps per (bin, species); warps take chunks of 32 particles in turn (chunk
+// c to warp c mod NW) and meet at a block barrier only at the end.
+//
+// What bounds it is instruction issue (the state's 56 bytes a particle alone take 0.27 ms
+// at 32.6M particles), so the pass over the chunks does only what every particle needs:
+// kick, drift, and the test that it is still in the bin.  A particle that is (about 94 %
+// on the 64^3 sphere) is written back to its own slot and deposits; in a bin that the
+// object cannot reach and that touches no reflecting face no other test is due.  Any other
+// particle only leaves its slot number in its warp's list, and 32 of them at a time go
+// through the whole push again (push_leavers: reflection, faces, object, hit cell, mover
+// list), so that the rare paths run on full warps.  The slots they leave are filled at the
+// end from the bin's last stayers, matched by their ranks over the chunks' stayer masks.
+// Against the pass that tested every particle for everything and compacted the stayers in
+// order (a look-back over the chunks' counts), one launch of 32.6M particles (64^3 cells,
+// bins of 4,096) went from 522 to 326 warp instructions a chunk and from 0.600 to 0.416 ms:
+// 0.65 of the measured copy rate for the 56 bytes a particle, 0.56 on the 160 x 160 x 80
+// crater (8.2 -> 5.8 ms).  Issue slots are then 67 % taken and the shared-memory pipe 60 %.
+//
+// A warp's next PUSH_DEPTH chunks are in flight at any time: one lane copies a chunk's 896
+// bytes into the warp's stage with a bulk copy (bins start on whole groups of 32 slots), so
+// the particles cost no address arithmetic and no registers while they travel.
 // HYBRID: the IFE mesh is finer than the PIC mesh, stayers deposit straight
 // onto its nodes (a separate instantiation keeps the common path's registers)
-constexpr int PUSH_WARPS = 8;   // 256 threads
 constexpr int PUSH_DEPTH = 3;   // chunks in flight per warp
+constexpr int PUSH_CHUNKS = (BIN_MAX + 31) / 32;
 
-// the push's dynamic shared memory for bins of edge B: node-field tile, deposit
-// tile, chunk counts, cp.async stages (in that order; every part a multiple of 16 bytes)
-template <int B>
+// the push's dynamic shared memory for bins of edge B: node-field pairs, deposit tile (first
+// the landing place of the node-field tile), stages, stayer masks (in that order).  The
+// stages' room later holds the masks' prefix counts and the list of slots to fill.
+// 16 deposit copies a node halve the atomics' bank conflicts against 8 (32, without any, were
+// no faster at 4,096 particles a bin and slower at 1,024); at B = 8 they would take 47 KB.
+template <int B, int NW>
 struct PushSmem {
     static constexpr int TL = B + 1, TN = TL * TL * TL;
-    static constexpr size_t et = sizeof(float4) * TN;
-    static constexpr size_t wt = sizeof(unsigned) * 8 * TN;
-    static constexpr size_t agg = sizeof(int) * ((((BIN_MAX + 31) / 32) + 3) & ~3);
-    static constexpr size_t stg = sizeof(unsigned) * PUSH_WARPS * PUSH_DEPTH * 7 * 32;
-    static constexpr size_t bytes = et + wt + agg + stg;
-    static_assert(et % 16 == 0 && wt % 16 == 0 && agg % 16 == 0, "16-byte parts");
+    static constexpr int NC = B == 4 ? 16 : 8;
+    static constexpr size_t pp = sizeof(float4) * TN, pq = (pp + sizeof(float2) * TN + 127) / 128 * 128;
+    static constexpr size_t wt = (sizeof(unsigned) * NC * TN + 127) / 128 * 128;
+    static constexpr size_t stg = sizeof(unsigned) * NW * PUSH_DEPTH * 7 * 32;
+    static constexpr size_t mask = sizeof(unsigned) * PUSH_CHUNKS;
+    static constexpr size_t bytes = pq + wt + stg + mask;
+    static constexpr int holes = (int)((stg - mask) / sizeof(unsigned short));   // slots to fill at a time
+    static_assert(mask % 16 == 0 && stg > mask, "the prefix counts fit in the stages");
+    static_assert(sizeof(float4) * TN <= wt, "the node-field tile lands in the deposit tile's room");
 };
 
-template <bool HYBRID, int B>
-__global__ void __launch_bounds__(256, 5) k_push_bins_m(Launch L, ObjF of, float dthf,
-                                                     const __grid_constant__ CUtensorMap tmE) {
-    using SM = PushSmem<B>;
+// no point of the box [x0, x1) x [y0, y1) x [z0, z1) is in the object, with a margin
+// above the FP32 level set's rounding
+PF_D bool box_clear(const ObjF& o, float x0, float x1, float y0, float y1, float z0, float z1) {
+    if (o.kind == 1) {
+        const float dx = fmaxf(fmaxf(x0 - o.a0, o.a0 - x1), 0.0f), dy = fmaxf(fmaxf(y0 - o.a1, o.a1 - y1), 0.0f),
+                    dz = fmaxf(fmaxf(z0 - o.a2, o.a2 - z1), 0.0f);
+        return dx * dx + dy * dy + dz * dz > o.a3 * 1.0001f + 0.01f;
+    } else if (o.kind == 2) {          // nothing of a cap crater lies above its ground
+        return z0 > o.a0 + 0.01f;
+    } else if (o.kind == 3) {
+        const float l = fminf(o.a0 * x0, o.a0 * x1) + fminf(o.a1 * y0, o.a1 * y1) + fminf(o.a2 * z0, o.a2 * z1);
+        const float big = fmaxf(fabsf(o.a0) * x1 + fabsf(o.a1) * y1 + fabsf(o.a2) * z1, fabsf(o.a3));
+        return l - o.a3 > 1e-4f * big + 0.01f;
+    } else if (o.kind == 4) {          // nor of a raised-rim crater above its rim (its floor is lower)
+        return z0 > fmaxf(o.a6, o.a11) + 0.01f;
+    }
+    return true;
+}
+
+// the whole push of up to 32 particles of the bin that did not simply stay in it (act: the
+// lanes that have one, in slot start + i): as push_one, then the survivors go to the mover
+// list and deposit in the rebin, with every mover of the step
+template <int TL>
+static __device__ __noinline__ void push_leavers(const Launch& L, const SpeciesDev& S, const ObjF& of, float dthf,
+                                                 const float4* P, const float2* Q, int x0, int y0, int z0, long long g,
+                                                 bool act, unsigned* sctr) {
+    int code = NONE, acc = -1;
+    PF32 p;
+    long long id = 0;
+    if (act) {
+        load_p(S.binsF, g, p);
+        if (L.track) id = S.binsF.id[g];
+        struct Tile {             // (a node as the neighbour of the one before it, but for the first of a row)
+            const float4* P;
+            const float2* Q;
+            int x0, y0, z0;
+            PF_D float4 operator()(int i, int j, int k) const {
+                const int second = i > x0, t = tile_index<TL>(i - second, j, k, x0, y0, z0);
+                const float4 p = P[t];
+                const float2 q = Q[t];
+                return second ? make_float4(p.y, p.w, q.y, 0.0f) : make_float4(p.x, p.z, q.x, 0.0f);
+            }
+        };
+        code = push_one(L, of, (float)S.k, dthf, S.reflect, p, Tile{P, Q, x0, y0, z0}, acc);
+        if (code == COLLECTED && acc >= 0) atomicAdd(&S.surf[acc], 1ull);
+    }
+    count_event32(&sctr[C_ABSORBED], code == ABSORBED);
+    count_event32(&sctr[C_COLLECTED], code == COLLECTED);
+    count_event32(&sctr[C_LOST], code == COLLECTED && acc < 0);
+    const bool alive = code == ALIVE;
+    const long long slot = warp_reserve(S.mov_out_n, alive);
+    if (alive) {
+        if (slot < S.mcap) store_p(S.movF_out, slot, p, id, L.track);
+        else atomicAdd(&S.ctr[C_DROPPED], 1ull);
+    }
+}
+
+// a bulk copy to shared memory, counted on an mbarrier
+PF_D void bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+template <bool HYBRID, int B, int NW>
+__global__ void __launch_bounds__(32 * NW, 32 / NW) k_push_bins_m(const __grid_constant__ Launch L, const __grid_constant__ ObjF of,
+                                                     float dthf, const __grid_constant__ CUtensorMap tmE) {
+    using SM = PushSmem<B, NW>;
+    constexpr int NT = 32 * NW;
     constexpr int TL = SM::TL, TN = SM::TN;
     extern __shared__ __align__(128) unsigned char push_smem[];
-    float4* Et = reinterpret_cast<float4*>(push_smem);   // the bin's node-field tile (TMA destination)
-    // deposits of the bin's stayers in units of 2^-19 particle, 8 interleaved
-    // copies per node (copy = lane & 7) so that the lanes of one atomic
+    float4* Ep = reinterpret_cast<float4*>(push_smem);   // the bin's node field in pairs along x
+    float2* Eq = reinterpret_cast<float2*>(push_smem + SM::pp);
+    // deposits of the bin's stayers in units of 2^-19 particle, NC interleaved
+    // copies per node (copy = lane % NC) so that the lanes of one atomic
     // instruction spread over the banks.  A particle adds 7 rounded weights and
     // the remainder 2^19 - sum (at least -4), so a copy, reached by at most
     // BIN_MAX / 8 + 1 particles, holds a value in [-2^14, 2^31]: exact in 32
     // bits modulo 2^32.  The flush multiplies by 2^13 (2^32 units per particle).
-    unsigned* Wt = reinterpret_cast<unsigned*>(push_smem + SM::et);
-    // stayers of chunk c plus one, for each chunk c (0: not yet published)
-    int* agg = reinterpret_cast<int*>(push_smem + SM::et + SM::wt);
-    __shared__ int s_total, s_fail;   // stayers of the bin plus one; a wait gave up
+    unsigned* Wt = reinterpret_cast<unsigned*>(push_smem + SM::pq);
+    float4* Et = reinterpret_cast<float4*>(Wt);          // the node-field tile (TMA destination) before
     // per warp and stage: cell, fx, fy, fz, vx, vy, vz of 32 particles
     typedef unsigned Stage[PUSH_DEPTH][7][32];
-    Stage* stg = reinterpret_cast<Stage*>(push_smem + SM::et + SM::wt + SM::agg);
-    __shared__ alignas(8) unsigned long long bar;
+    Stage* stg = reinterpret_cast<Stage*>(push_smem + SM::pq + SM::wt);
+    unsigned* stay_mask = reinterpret_cast<unsigned*>(push_smem + SM::pq + SM::wt + SM::stg);   // [chunk]
+    __shared__ alignas(8) unsigned long long bar, sbar[NW][PUSH_DEPTH];
     __shared__ unsigned sctr[NCTR];
-    __shared__ int s_ok;
+    __shared__ unsigned short list[NW][64];   // slots that wait for push_leavers, per warp
+    __shared__ unsigned short rest[NW * 32];  // what the warps have left over at the end
+    __shared__ int s_ok, s_rest, s_sum[NW];
     const int s = blockIdx.y;
     const int b = blockIdx.x;
     const SpeciesDev& S = L.sp[s];
@@ -378,36 +464,32 @@ __global__ void __launch_bounds__(256, 5) k_push_bins_m(Launch L, ObjF of, float
     }
     const int bx = b % L.nbx, by = (b / L.nbx) % L.nby, bz = b / (L.nbx * L.nby);
     const int x0 = bx * B, y0 = by * B, z0 = bz * B;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nch = (n + 31) >> 5;
     const long long start = S.bstart[b];
-    // copies of chunk cc (this warp's) into stage slot sl; one group per call
+    unsigned* const bin = S.binsF.w + (start >> 5) * PGROUP;   // (bins start on whole groups)
+    // one lane copies chunk cc (this warp's) into stage slot sl
     auto stage = [&](int cc, int sl) {
-        const int ii = cc * 32 + lane;
-        if (cc < nch && ii < n) {
-            const long long g = start + ii;
-            unsigned(&d)[7][32] = stg[wid][sl];
-            cp_async4(&d[0][lane], S.binsF.cell + g);
-            cp_async4(&d[1][lane], S.binsF.fx + g);
-            cp_async4(&d[2][lane], S.binsF.fy + g);
-            cp_async4(&d[3][lane], S.binsF.fz + g);
-            cp_async4(&d[4][lane], S.binsF.vx + g);
-            cp_async4(&d[5][lane], S.binsF.vy + g);
-            cp_async4(&d[6][lane], S.binsF.vz + g);
+        if (cc < nch && lane == 0) {
+            mbar_expect_tx(&sbar[wid][sl], 4 * PGROUP);
+            bulk_copy(stg[wid][sl], bin + cc * PGROUP, 4 * PGROUP, &sbar[wid][sl]);
         }
-        cp_async_commit();
     };
-#pragma unroll
-    for (int d = 0; d < PUSH_DEPTH; ++d) stage(wid + d * nw, d);
-    if (tid == 0) { mbar_init(&bar, 1); fence_barrier_init(); }
-    for (int t = tid; t < 8 * TN; t += blockDim.x) Wt[t] = 0u;
-    for (int t = tid; t < nch; t += blockDim.x) agg[t] = 0;
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        for (int q = 0; q < NW * PUSH_DEPTH; ++q) mbar_init(&sbar[0][q], 1);
+        fence_barrier_init();
+        s_rest = 0;
+    }
     if (tid < NCTR) sctr[tid] = 0u;
-    if (tid == 0) { s_total = 0; s_fail = 0; }
     __syncthreads();
     if (tid == 0) {
         mbar_expect_tx(&bar, TN * (unsigned)sizeof(float4));
         tma_load_4d(Et, &tmE, &bar, 0, x0, y0, z0);
+    }
+#pragma unroll
+    for (int d = 0; d < PUSH_DEPTH; ++d) stage(wid + d * NW, d);
+    if (tid == 0) {
         bool ok = mbar_wait_bounded(&bar, 0);
         if (!ok) {
             atomicOr(L.err, ERR_TMA_TIMEOUT);
@@ -416,121 +498,193 @@ __global__ void __launch_bounds__(256, 5) k_push_bins_m(Launch L, ObjF of, float
         s_ok = ok;
     }
     __syncthreads();
-    if (!s_ok) {   // (the bin is left as it was; the error flag reports it)
-        cp_async_wait_all();
-        if (tid == 0) S.bstay[b] = n;
-        return;
-    }
-    const bool track = L.track;
+    for (int t = tid; t < TN; t += NT)
+        if (t % TL < TL - 1) {
+            const float4 u = Et[t], v = Et[t + 1];
+            Ep[t] = make_float4(u.x, v.x, u.y, v.y);
+            Eq[t] = make_float2(u.z, v.z);
+        }
+    __syncthreads();
+    for (int t = tid; t < SM::NC * TN; t += NT) Wt[t] = 0u;
+    __syncthreads();
     const float kf = (float)S.k;
-    const int refl = S.reflect;
-    const int copy = lane & 7;
-    volatile int* vagg = agg;
-    volatile int* vfail = &s_fail;
-    int run = 0;   // stayers of chunks 0..c-nw (this warp's previous chunk included)
-    unsigned c_push = 0, c_abs = 0, c_col = 0, c_lost = 0;
-    int sl = 0;   // stage slot of the current chunk
-    for (int c = wid; c < nch; c += nw) {
+    // the bin's cells inside the mesh, the reflecting faces it touches, and whether the
+    // object reaches it
+    const int lx = min(B, L.mesh.nx - x0), ly = min(B, L.mesh.ny - y0), lz = min(B, L.mesh.nz - z0);
+    const int refl = S.reflect & ((x0 == 0 ? 1 : 0) | (x0 + lx == L.mesh.nx ? 2 : 0) | (y0 == 0 ? 4 : 0) |
+                                  (y0 + ly == L.mesh.ny ? 8 : 0) | (z0 == 0 ? 16 : 0) | (z0 + lz == L.mesh.nz ? 32 : 0));
+    const bool clear = box_clear(of, (float)x0, (float)(x0 + lx), (float)y0, (float)(y0 + ly), (float)z0, (float)(z0 + lz));
+    const int cell0 = pack_cell(x0, y0, z0);
+    const int copy = lane & (SM::NC - 1);
+    unsigned short* mine = list[wid];
+    int waiting = 0;                       // slots in this warp's list
+    bool fail = !s_ok;
+    int sl = 0;                            // stage slot of the current chunk
+    unsigned phase = 0;                    // its parity
+    for (int c = wid; c < nch; c += NW) {
         const int i = c * 32 + lane;
-        int code = NONE, acc = -1;
-        PF32 p;
-        long long id = 0;
-        cp_async_wait<PUSH_DEPTH - 1>();   // this chunk's group (each lane reads only its own copies)
-        {
-            const unsigned(&d)[7][32] = stg[wid][sl];
-            unpack_cell((int)d[0][lane], p.i, p.j, p.k);
-            p.fx = __uint_as_float(d[1][lane]); p.fy = __uint_as_float(d[2][lane]);
-            p.fz = __uint_as_float(d[3][lane]); p.vx = __uint_as_float(d[4][lane]);
-            p.vy = __uint_as_float(d[5][lane]); p.vz = __uint_as_float(d[6][lane]);
+        const bool live = i < n;
+        if (!mbar_try_wait(&sbar[wid][sl], phase) && !mbar_wait_bounded(&sbar[wid][sl], phase)) {
+            if (lane == 0) atomicOr(L.err, ERR_TMA_TIMEOUT);
+            fail = true;
         }
-        if (track && i < n) id = S.binsF.id[start + i];
-        if (i < n) {
-            // kick with the field gathered at the old position, then drift
-            const WF w = weights_f(p.fx, p.fy, p.fz);
-            float ex, ey, ez;
-            gather_tile<TL>(Et, tile_index<TL>(p.i, p.j, p.k, x0, y0, z0), w, ex, ey, ez);
-            p.vx += kf * ex; p.vy += kf * ey; p.vz += kf * ez;
-            const float xo = (float)p.i + p.fx, yo = (float)p.j + p.fy, zo = (float)p.k + p.fz;
-            p.fx += p.vx * dthf; p.fy += p.vy * dthf; p.fz += p.vz * dthf;
-            advance_axis(p.fx, p.i); advance_axis(p.fy, p.j); advance_axis(p.fz, p.k);
-            if (refl) reflect_cell(L.mesh, refl, p);
-            if (p.i < 0 || p.i >= L.mesh.nx || p.j < 0 || p.j >= L.mesh.ny || p.k < 0 || p.k >= L.mesh.nz) {
-                code = ABSORBED;
-            } else {
-                const float xn = (float)p.i + p.fx, yn = (float)p.j + p.fy, zn = (float)p.k + p.fz;
-                if (level_set_f(of, xn, yn, zn) < 0.0f) {
-                    acc = hit_cell_f(L, of, xo, yo, zo, xn, yn, zn);
-                    code = COLLECTED;
-                } else {
-                    code = ALIVE;
-                }
+        if (fail) {   // (one more bounded wait for each copy in flight, so that none lands after the block has left)
+            for (int d = 0; d < PUSH_DEPTH && c + d * NW < nch; ++d) {
+                mbar_wait_bounded(&sbar[wid][sl], phase);
+                if (++sl == PUSH_DEPTH) { sl = 0; phase ^= 1; }
             }
-        }
-        // refill the slot (its values have been used, so its reads are done)
-        stage(c + PUSH_DEPTH * nw, sl);
-        sl = sl + 1 == PUSH_DEPTH ? 0 : sl + 1;
-        bool stay = false, mover = false;
-        if (code == ALIVE) {
-            stay = (p.i >= x0) & (p.i < x0 + B) & (p.j >= y0) & (p.j < y0 + B) & (p.k >= z0) & (p.k < z0 + B);
-            mover = !stay;
-            if (HYBRID && stay) {
-                global_deposit_f(L, S.W, p);   // hybrid grid: straight onto the IFE nodes
-            } else if (stay) {   // (movers deposit in the rebin, with every mover of the step)
-                tile_deposit19<TL>(Wt, 8 * tile_index<TL>(p.i, p.j, p.k, x0, y0, z0) + copy, weights_f(p.fx, p.fy, p.fz));
-            }
-        } else if (code == COLLECTED) {
-            if (acc >= 0) atomicAdd(&S.surf[acc], 1ull);
-        }
-        c_push += code != NONE;
-        c_abs += code == ABSORBED;
-        c_col += code == COLLECTED;
-        c_lost += code == COLLECTED && acc < 0;
-        // publish this chunk's count, then add those of chunks c-7..c-1 (bounded waits)
-        const unsigned bal = __ballot_sync(0xffffffffu, stay);
-        if (lane == 0) vagg[c] = __popc(bal) + 1;
-        unsigned got = 0;
-        bool ok = true;
-        if (lane >= 1 && lane < nw && c - lane >= 0) {
-            int v;
-            long long spins = 0;
-            while ((v = vagg[c - lane]) == 0)
-                if (++spins > (1ll << 26) || *vfail) { ok = false; break; }
-            got = ok ? (unsigned)(v - 1) : 0u;
-        }
-        if (!__all_sync(0xffffffffu, ok)) {   // give up: this bin's stayers are dropped
-            if (lane == 0) { *vfail = 1; atomicOr(L.err, ERR_CHUNK_TIMEOUT); }
             break;
         }
-        const int before = run + (int)__reduce_add_sync(0xffffffffu, got);
-        run = before + __popc(bal);
-        if (lane == 0 && c == nch - 1) s_total = run + 1;
-        if (stay) store_p(S.binsF, start + before + __popc(bal & ((1u << lane) - 1)), p, id, track);
-        long long slot = warp_reserve(S.mov_out_n, mover);
-        if (mover) {
-            if (slot < S.mcap) store_p(S.movF_out, slot, p, id, track);
-            else atomicAdd(&S.ctr[C_DROPPED], 1ull);
+        // the cell relative to the bin, until the end
+        int ri, rj, rk;
+        float fx, fy, fz, vx, vy, vz;
+        {
+            const unsigned(&d)[7][32] = stg[wid][sl];
+            unpack_cell(live ? (int)d[0][lane] : cell0, ri, rj, rk);
+            ri -= x0; rj -= y0; rk -= z0;
+            fx = __uint_as_float(d[1][lane]); fy = __uint_as_float(d[2][lane]); fz = __uint_as_float(d[3][lane]);
+            vx = __uint_as_float(d[4][lane]); vy = __uint_as_float(d[5][lane]); vz = __uint_as_float(d[6][lane]);
+        }
+        // kick with the field gathered at the old position, then drift
+        {
+            const WF w = weights_f(fx, fy, fz);
+            float ex, ey, ez;
+            gather_tile<TL>(Ep, Eq, ri + TL * (rj + TL * rk), w, ex, ey, ez);
+            vx += kf * ex; vy += kf * ey; vz += kf * ez;
+        }
+        fx += vx * dthf; fy += vy * dthf; fz += vz * dthf;
+        advance_axis(fx, ri); advance_axis(fy, rj); advance_axis(fz, rk);
+        if (refl) {
+            PF32 p{ri + x0, rj + y0, rk + z0, fx, fy, fz, vx, vy, vz};
+            reflect_cell(L.mesh, refl, p);
+            ri = p.i - x0; rj = p.j - y0; rk = p.k - z0;
+            fx = p.fx; fy = p.fy; fz = p.fz; vx = p.vx; vy = p.vy; vz = p.vz;
+        }
+        bool stay = live & ((unsigned)ri < (unsigned)lx) & ((unsigned)rj < (unsigned)ly) & ((unsigned)rk < (unsigned)lz);
+        if (!clear)
+            stay = stay &&
+                   !(level_set_f(of, (float)(ri + x0) + fx, (float)(rj + y0) + fy, (float)(rk + z0) + fz) < 0.0f);
+        const unsigned bal = __ballot_sync(0xffffffffu, stay);
+        // refill the stage slot: the bulk copy is not ordered after the reads of the slot by
+        // itself, but the vote above has waited for what every lane made of its seven words
+        stage(c + PUSH_DEPTH * NW, sl);
+        if (++sl == PUSH_DEPTH) { sl = 0; phase ^= 1; }
+        if (stay) {
+            unsigned* o = bin + (c * PGROUP + lane);
+            o[0] = (unsigned)(cell0 + ri + (rj << 11) + (rk << 22));
+            o[32] = __float_as_uint(fx); o[64] = __float_as_uint(fy); o[96] = __float_as_uint(fz);
+            o[128] = __float_as_uint(vx); o[160] = __float_as_uint(vy); o[192] = __float_as_uint(vz);
+            if (HYBRID) {          // hybrid grid: straight onto the IFE nodes
+                global_deposit_f(L, S.W, PF32{ri + x0, rj + y0, rk + z0, fx, fy, fz, vx, vy, vz});
+            } else {               // (movers deposit in the rebin, with every mover of the step)
+                tile_deposit19<TL, SM::NC>(Wt, SM::NC * (ri + TL * (rj + TL * rk)) + copy, fx, fy, fz);
+            }
+        }
+        if (lane == 0) stay_mask[c] = bal;
+        const unsigned gone = __ballot_sync(0xffffffffu, live && !stay);
+        if (gone) {
+            if (live && !stay) mine[waiting + __popc(gone & ((1u << lane) - 1))] = (unsigned short)i;
+            waiting += __popc(gone);
+            __syncwarp();
+            if (waiting >= 32) {
+                push_leavers<TL>(L, S, of, dthf, Ep, Eq, x0, y0, z0, start + mine[lane], true, sctr);
+                waiting -= 32;
+                const unsigned short up = mine[32 + lane];
+                __syncwarp();
+                mine[lane] = up;
+                __syncwarp();
+            }
         }
     }
-    cp_async_wait_all();   // (a warp that gave up may still have copies in flight)
+    // what the warps have left, 32 to a warp again
+    {
+        int at = 0;
+        if (lane == 0 && waiting) at = atomicAdd(&s_rest, waiting);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (lane < waiting) rest[at + lane] = mine[lane];
+    }
+    // (a warp that gave up: the bin's particles are dropped, the error flag reports it; a
+    // tile that never came: the bin is left as it was)
+    if (__syncthreads_or(fail)) {
+        if (tid == 0) {
+            const int left = s_ok ? 0 : n;
+            S.bcount[b] = left;
+            S.bstay[b] = left;
+        }
+        return;
+    }
+    for (int q = wid * 32; q < s_rest; q += NW * 32) {
+        const bool act = q + lane < s_rest;
+        push_leavers<TL>(L, S, of, dthf, Ep, Eq, x0, y0, z0, start + (act ? (int)rest[q + lane] : 0), act, sctr);
+    }
+    // the stayers' count before each chunk
+    int* pre = reinterpret_cast<int*>(stg);
+    int total;
+    {
+        constexpr int PER = (PUSH_CHUNKS + NT - 1) / NT;
+        int cnt[PER], sum = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c_push += __shfl_xor_sync(0xffffffffu, c_push, o);
-        c_abs += __shfl_xor_sync(0xffffffffu, c_abs, o);
-        c_col += __shfl_xor_sync(0xffffffffu, c_col, o);
-        c_lost += __shfl_xor_sync(0xffffffffu, c_lost, o);
+        for (int q = 0; q < PER; ++q) {
+            cnt[q] = tid * PER + q < nch ? __popc(stay_mask[tid * PER + q]) : 0;
+            sum += cnt[q];
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane == 31) s_sum[wid] = inc;
+        __syncthreads();
+        int run = inc - sum;
+        total = 0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            if (q < wid) run += s_sum[q];
+            total += s_sum[q];
+        }
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (tid * PER + q < nch) pre[tid * PER + q] = run;
+            run += cnt[q];
+        }
     }
-    if (lane == 0) {
-        if (c_push) atomicAdd(&sctr[C_PUSHED], c_push);
-        if (c_abs) atomicAdd(&sctr[C_ABSORBED], c_abs);
-        if (c_col) atomicAdd(&sctr[C_COLLECTED], c_col);
-        if (c_lost) atomicAdd(&sctr[C_LOST], c_lost);
+    __syncthreads();   // (also: the leavers have been read from their slots)
+    // the stayers in slots from `total` on move to the slots below it that leavers left,
+    // in order of their ranks, SM::holes at a time
+    unsigned short* hole = reinterpret_cast<unsigned short*>(push_smem + SM::pq + SM::wt + SM::mask);
+    const int c1 = total >> 5;
+    const int below = c1 < nch ? pre[c1] + __popc(stay_mask[c1] & ((1u << (total & 31)) - 1)) : total;
+    const unsigned lt = (1u << lane) - 1;
+    for (int h0 = 0; h0 < total - below; h0 += SM::holes) {
+        for (int c = tid; c * 32 < total; c += NT) {
+            unsigned m = ~stay_mask[c];
+            if (total - c * 32 < 32) m &= (1u << (total - c * 32)) - 1;
+            for (int rank = c * 32 - pre[c] - h0; m; ++rank, m &= m - 1)
+                if (rank >= 0 && rank < SM::holes) hole[rank] = (unsigned short)(c * 32 + __ffs(m) - 1);
+        }
+        __syncthreads();
+        for (int c = c1 + wid; c < nch; c += NW) {
+            const unsigned m = stay_mask[c];
+            const int slot = c * 32 + lane, rank = pre[c] + __popc(m & lt) - below - h0;
+            if (slot >= total && ((m >> lane) & 1) && rank >= 0 && rank < SM::holes) {
+                const int to = hole[rank];
+                unsigned* o = bin + pword(to);
+                const unsigned* f = bin + pword(slot);
+#pragma unroll
+                for (int d = 0; d < 7; ++d) o[32 * d] = f[32 * d];
+                if (L.track) S.binsF.id[start + to] = S.binsF.id[start + slot];
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
     if (tid == 0) {
-        S.bcount[b] = (s_fail || s_total == 0) ? 0 : s_total - 1;
-        S.bstay[b] = S.bcount[b];
+        S.bcount[b] = total;
+        S.bstay[b] = total;
+        sctr[C_PUSHED] = (unsigned)n;
     }
-    tile_flush19<TL>(L, S.W, Wt, x0, y0, z0);
+    tile_flush19<TL, SM::NC>(L, S.W, Wt, x0, y0, z0);
+    __syncthreads();
     if (tid < NCTR && sctr[tid]) atomicAdd(&S.ctr[tid], (unsigned long long)sctr[tid]);
 }
 
@@ -801,9 +955,7 @@ __global__ void k_half_kick_bins_m(Launch L) {
         load_p(S.binsF, st + i, p);
         float ex, ey, ez;
         gather_f(p.i, p.j, p.k, weights_f(p.fx, p.fy, p.fz), ea, ex, ey, ez);
-        S.binsF.vx[st + i] = p.vx - kh * ex;
-        S.binsF.vy[st + i] = p.vy - kh * ey;
-        S.binsF.vz[st + i] = p.vz - kh * ez;
+        store_v(S.binsF, st + i, p.vx - kh * ex, p.vy - kh * ey, p.vz - kh * ez);
     }
 }
 __global__ void k_half_kick_list_m(Launch L) {
@@ -816,9 +968,7 @@ __global__ void k_half_kick_list_m(Launch L) {
         load_p(S.movF_in, i, p);
         float ex, ey, ez;
         gather_f(p.i, p.j, p.k, weights_f(p.fx, p.fy, p.fz), ea, ex, ey, ez);
-        S.movF_in.vx[i] = p.vx - kh * ex;
-        S.movF_in.vy[i] = p.vy - kh * ey;
-        S.movF_in.vz[i] = p.vz - kh * ez;
+        store_v(S.movF_in, i, p.vx - kh * ex, p.vy - kh * ey, p.vz - kh * ez);
     }
 }
 
@@ -840,17 +990,32 @@ static InjArgs inj_args_m(Ctx& c) {
 __global__ void k_inject_counts(InjArgs a);   // particles.cu
 __global__ void k_step_advance(long long* step);
 
-// one push launch; the kernel's dynamic shared-memory limit is raised once
-// to what bins of edge B need (above the 48 KB default at B = 8)
-template <bool HYBRID, int B>
+// one push launch; the kernel's dynamic shared-memory limit is raised once to what it
+// needs (above the 48 KB default)
+template <bool HYBRID, int B, int NW>
 static cudaError_t push_bins_m(dim3 grid, cudaStream_t st, const Launch& L, const ObjF& of, float dthf,
                                const CUtensorMap& tm) {
-    static_assert(PushSmem<B>::bytes <= 200 * 1024, "push shared memory");
-    void* kern = (void*)k_push_bins_m<HYBRID, B>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PushSmem<B>::bytes);
+    using SM = PushSmem<B, NW>;
+    static_assert(SM::bytes <= 200 * 1024, "push shared memory");
+    void* kern = (void*)k_push_bins_m<HYBRID, B, NW>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
     if (e != cudaSuccess) return e;
-    k_push_bins_m<HYBRID, B><<<grid, 256, PushSmem<B>::bytes, st>>>(L, of, dthf, tm);
+    k_push_bins_m<HYBRID, B, NW><<<grid, 32 * NW, SM::bytes, st>>>(L, of, dthf, tm);
     return cudaGetLastError();
+}
+// Warps per block by the slots of a bin (particles and a quarter more, of the fullest
+// species).  A block spends about 8 us outside the pass over its chunks (tile, leavers,
+// filled slots, flush), so small bins want many small blocks in an SM to hide one's ends
+// behind the others, large ones long passes that many warps share.  Push of the 64^3 sphere
+// in ms: 4^3-cell bins of 512 particles 0.107 with 4 warps and 0.138 with 8, 2,048 0.236
+// and 0.255, 3,072 0.336 and 0.332, 8,000 0.901 and 0.790; 8^3-cell bins of 4,096 particles
+// 0.0944 with 8 warps and 0.0954 with 16, 8,192 0.151 and 0.143, 24,576 0.397 and 0.359.
+constexpr long long PUSH_SMALL = 3700, PUSH_LARGE = 6200;   // slots of a bin, at B = 4 and 8
+template <int B>
+static cudaError_t push_bins_by_fill(dim3 grid, cudaStream_t st, const Launch& L, const ObjF& of, float dthf,
+                                     const CUtensorMap& tm, long long slots) {
+    if (slots < (B == 4 ? PUSH_SMALL : PUSH_LARGE)) return push_bins_m<false, B, B == 4 ? 4 : 8>(grid, st, L, of, dthf, tm);
+    return push_bins_m<false, B, B == 4 ? 8 : 16>(grid, st, L, of, dthf, tm);
 }
 
 // what precedes a push: the step's mover-list counts and node charges start at zero
@@ -872,13 +1037,16 @@ cudaError_t launch_push_bins_mixed(Ctx& c) {
     const dim3 grid(c.nblocks, ns);
     const ObjF of = obj_f(c.obj);
     const float dthf = (float)c.dth;
+    long long slots = 0;
+    for (const Species& q : c.sp) slots = q.cap > slots ? q.cap : slots;
+    slots /= c.nblocks;
     cudaError_t e;
     if (c.bin_edge == 8)
-        e = c.refine == 1 ? push_bins_m<false, 8>(grid, c.stream, L, of, dthf, c.tmapEf)
-                          : push_bins_m<true, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
+        e = c.refine == 1 ? push_bins_by_fill<8>(grid, c.stream, L, of, dthf, c.tmapEf, slots)
+                          : push_bins_m<true, 8, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
     else
-        e = c.refine == 1 ? push_bins_m<false, 4>(grid, c.stream, L, of, dthf, c.tmapEf)
-                          : push_bins_m<true, 4>(grid, c.stream, L, of, dthf, c.tmapEf);
+        e = c.refine == 1 ? push_bins_by_fill<4>(grid, c.stream, L, of, dthf, c.tmapEf, slots)
+                          : push_bins_m<true, 4, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
     c.launches += 1;
     return e;
 }
@@ -1068,29 +1236,20 @@ cudaError_t launch_flatten_mixed_to_f64(Ctx& c, int s, PArr flat, unsigned long 
 }
 
 void free_parrf(PArrF& a) {
-    if (a.base) {
-        lib_free(a.base);
-    } else {
-        lib_free(a.cell); lib_free(a.fx); lib_free(a.fy); lib_free(a.fz); lib_free(a.vx); lib_free(a.vy);
-        lib_free(a.vz); lib_free(a.id);
-    }
+    lib_free(a.base);
     a = PArrF{};
 }
 
-// the seven 4-byte arrays (and 8-byte ids first, for their alignment) in one allocation
+// the groups of 32 particles, then the ids, in one allocation
 cudaError_t alloc_parrf(PArrF& a, long long n, bool id) {
     free_parrf(a);
-    const size_t m = (size_t)(n > 0 ? n : 1);
-    const size_t mid = id ? sizeof(long long) * m : 0;
+    const size_t groups = (size_t)(n > 0 ? n + 31 : 32) / 32;
     char* b = nullptr;
-    cudaError_t e = lib_malloc(&b, mid + 7 * sizeof(float) * m);
+    cudaError_t e = lib_malloc(&b, groups * (sizeof(unsigned) * PGROUP + (id ? sizeof(long long) * 32 : 0)));
     if (e != cudaSuccess) return e;
     a.base = b;
-    if (id) a.id = (long long*)b;
-    char* f = b + mid;
-    a.cell = (int*)f;
-    float** arr[6] = {&a.fx, &a.fy, &a.fz, &a.vx, &a.vy, &a.vz};
-    for (int d = 0; d < 6; ++d) *arr[d] = (float*)(f + sizeof(float) * m * (d + 1));
+    a.w = (unsigned*)b;
+    if (id) a.id = (long long*)(b + groups * sizeof(unsigned) * PGROUP);
     return cudaSuccess;
 }
 
