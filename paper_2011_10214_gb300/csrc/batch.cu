@@ -157,6 +157,12 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             continue;
         }
         csize[i] = cluster_size_for(c.mesh.nnodes, node_halo(c.mesh), mixed, b->cta_nodes);
+        if (mixed && csize[i] > 0 && b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx == 0 && !c.fd_wanted) {
+            // the plan on first use (and the member's own solve re-planned with it)
+            c.fd_wanted = true;
+            cudaError_t e = build_pcg_graph(c);
+            if (e != cudaSuccess) return e;
+        }
         if (csize[i] > 0 && uses_fd(b, c)) csize[i] = fd_cluster_size(c.mesh.nnodes, b->cta_nodes);
     }
     const int groups[6] = {16, 8, 4, 2, 1, 0};

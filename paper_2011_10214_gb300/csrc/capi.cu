@@ -69,6 +69,7 @@ void free_mg(Ctx& c);                         // pcg_mg.cu
 void free_fd(Ctx& c);                         // pcg_fd.cu
 cudaError_t build_pcg_graph(Ctx& c);          // field.cu
 cudaError_t last_solve_converged(Ctx& c, bool* conv);
+cudaError_t move_to_fd(Ctx& c);
 
 // 5-tet split tables, computed from the definition (reading of Sec. 3.1.1)
 static TetTables make_tables() {
@@ -1089,14 +1090,14 @@ static pifepic_status settle_solver(pifepic_ctx* ctx) {
     const bool capped = !c.last_conv && c.last_iters >= c.maxit;
     if (c.solves_done < 2 || !(capped || c.last_conv)) return PIFEPIC_OK;
     if (c.fd_ready && !c.fd_single) {
-        c.fd_now = true;
-    } else if (capped && !c.mg_escalated) {
-        c.fd_capped = c.fd_single;
-        c.mg_escalated = true;
-    } else {
+        CUDA_OK(move_to_fd(c));
         return PIFEPIC_OK;
     }
-    CUDA_OK(build_pcg_graph(c));
+    if (capped && !c.mg_escalated) {
+        c.fd_capped = c.fd_single;
+        c.mg_escalated = true;
+        CUDA_OK(build_pcg_graph(c));
+    }
     return PIFEPIC_OK;
 }
 // the same inside a long call, at its step FD_LOOK: moves on if the last solve
@@ -1109,8 +1110,7 @@ static cudaError_t settle_inside(Ctx& c, int steps_done) {
     bool conv = false;
     cudaError_t e = last_solve_converged(c, &conv);   // (waits for the stream)
     if (e != cudaSuccess || !conv) return e;
-    c.fd_now = true;
-    return build_pcg_graph(c);
+    return move_to_fd(c);
 }
 
 pifepic_status pifepic_solve(pifepic_ctx* ctx, pifepic_stats* st) {

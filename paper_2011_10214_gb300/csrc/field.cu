@@ -428,8 +428,7 @@ int solve_graph_fixed_kernels(const Ctx& c) { return (c.ncut > 0) + (c.nit > 0) 
 
 // The solve as one CUDA graph (both precisions): q_T -> RHS -> warm start ->
 // persistent PCG -> node field
-cudaError_t build_pcg_graph(Ctx& c) {
-    plan_pcg(c);
+static cudaError_t capture_pcg_graph(Ctx& c) {
     if (c.pcg_exec) { cudaGraphExecDestroy(c.pcg_exec); c.pcg_exec = nullptr; }
     if (c.pcg_graph) { cudaGraphDestroy(c.pcg_graph); c.pcg_graph = nullptr; }
     cudaStream_t cs;
@@ -447,6 +446,17 @@ cudaError_t build_pcg_graph(Ctx& c) {
     else if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
     return e;
+}
+
+cudaError_t build_pcg_graph(Ctx& c) {
+    plan_pcg(c);
+    return capture_pcg_graph(c);
+}
+
+// the context's solves move on to the fast-diagonalisation PCG (its plan stands)
+cudaError_t move_to_fd(Ctx& c) {
+    c.fd_now = c.fd_single = true;
+    return capture_pcg_graph(c);
 }
 
 static cudaError_t set_pcg_state(Ctx& c) {

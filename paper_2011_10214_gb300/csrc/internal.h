@@ -122,7 +122,10 @@ struct PhotoDev {
     int ntri, acc;                  // triangles; cut-cell accumulator of the tet's cell
 };
 constexpr int PHOTO_RATE_BITS = 20;  // per-tet rates and carries in units of 2^-20 particles
-constexpr int BAR64_WORDS = 160;     // PCG exchange words per context (Ctx::bar64): 10 lines of 16
+// PCG exchange words per context (Ctx::bar64): 10 lines of 16, and 4 more for the
+// fast-diagonalisation PCG, whose grid may be another one (a counter holds a multiple of
+// the grid size between launches)
+constexpr int BAR64_FD = 160, BAR64_WORDS = 224;
 
 struct Launch {                     // what every particle kernel needs
     Mesh mesh;
@@ -283,6 +286,7 @@ struct Ctx {
     bool mg_escalated = false;        // AUTO: a Jacobi solve ended at the cap unconverged; another solver since
     bool fd_capped = false;           // AUTO: a fast-diagonalisation solve did; multigrid since
     FdPlan fd;                        // fast-diagonalisation preconditioner (fd.mx = 0: none)
+    bool fd_wanted = false;           // a batch solves this context with it: plan it on a smaller mesh too
     bool fd_ready = false;            // pifepic_solve_field uses it
     bool fd_now = false;              // a warm-started Jacobi solve is done: the steps use it too
     bool fd_single = false;           // the solves of pifepic_solve and pifepic_step use it

@@ -887,7 +887,7 @@ cudaError_t plan_pcg_fd(Ctx& c) {
     free_fd(c);
     const Mesh& m = c.mesh;
     if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || c.fd_capped ||
-        m.nnodes < FD_CLUSTER_MIN_NODES)
+        m.nnodes < (c.fd_wanted ? FD_CLUSTER_MIN_NODES : FD_MIN_NODES))
         return cudaSuccess;
     int dir[6], any = 0;
     for (int f = 0; f < 6; ++f) any |= dir[f] = c.bc[f].kind == PIFEPIC_BC_DIRICHLET;
@@ -1004,8 +1004,8 @@ static FdArgs fd_args(Ctx& c) {
     a.margin2 = c.inner_margin * c.inner_margin;
     a.maxit = 0;
     a.val = c.coop_partial;
-    a.arrivals = c.bar64;
-    a.fx = c.bar64 + FX_LINE;
+    a.arrivals = c.bar64 + BAR64_FD;
+    a.fx = c.bar64 + BAR64_FD + FX_LINE;
     a.hold = (const int*)(c.scal + 45);
     a.S = (PcgState*)c.scal;
     a.it_total = (long long*)(c.scal + 40);

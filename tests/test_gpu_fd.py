@@ -108,6 +108,27 @@ def test_steps_move_to_fast_diagonal_after_a_warm_solve(steps):
         gpu.close()
 
 
+def test_field_solves_between_steps():
+    """pifepic_solve_field runs the fast-diagonalisation PCG from the start; its solves
+    do not disturb those of the steps around it, before and after they move on."""
+    n, bc = (33, 32, 34), [D] * 6
+    gpu, orc = _pair(n, bc, _sphere(n))
+    add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+    explicit_particles(gpu, orc, 0, 3000, 7, 0.5)
+    g = np.random.default_rng(9)
+    for k in range(4):
+        F = g.normal(size=orc.fs.mesh.nnodes) * orc.fs.mesh.h ** 3
+        phi, _, _ = orc.fs.solve(F, np.zeros(len(orc.fs.it_cell)), tol=1e-12, maxit=5000)
+        gpu.solve_field(F)
+        assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max()
+        gpu.solve() if k == 0 else gpu.step(1)
+        F = gpu.node_charge(0) * (-0.01 / 2.0 ** 32)
+        qT = orc.fs.q_tets(-0.01 * gpu.surface_counts(0).astype(np.float64))
+        phi, _, _ = orc.fs.solve(F, qT, tol=1e-12, maxit=5000)
+        assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max(), k
+    gpu.close()
+
+
 # members of a batch: clusters of 2 to 16 CTAs, a CTA's planes transformed in groups; every pair of ends, one free
 # node along an axis, z runs of 16 rows
 BATCH = [((13, 12, 14), [D] * 6), ((17, 16, 15), [N, D, D, D, N, D]), ((24, 33, 9), [D, D, N, N, D, N]),
