@@ -369,8 +369,7 @@ pifepic_status pifepic_create(const pifepic_mesh_desc* mesh, const pifepic_solve
     ALLOC(c.red_ticket, sizeof(unsigned) * 4);
     ALLOC(c.bar64, sizeof(unsigned long long) * BAR64_WORDS);
     ALLOC(c.err_word, sizeof(int));
-    ALLOC(c.stat_dev, sizeof(StatPack));
-    if (cudaMallocHost(&c.stat_host, sizeof(StatPack)) != cudaSuccess) {
+    if (cudaMallocHost(&c.stat_host, 2 * sizeof(StatPack)) != cudaSuccess) {
         cudaGetLastError();
         c.stat_host = nullptr;
         FAIL(PIFEPIC_ENOMEM, "pinned statistics buffer");
@@ -414,7 +413,7 @@ void pifepic_destroy(pifepic_ctx* ctx) {
                     c.z ? (void*)(c.z - c.zguard) : nullptr, c.zf ? (void*)(c.zf - c.zguard) : nullptr,
                     c.rf, c.pf, c.qf, c.uf, c.E, c.Ef, c.Wall, c.surfall, c.ctrall, c.imask, c.ibase, c.cell_acc,
                     c.it_cell, c.it_t, c.it_data, c.it_acc, c.qT, c.cut_cell, c.cut_area, c.qcut, c.patch_node,
-                    c.patch_coef, c.patch_coeff, c.red, c.coop_partial, c.rowkind, c.pcg_x, c.ph_tets, c.ph_Q, c.ph_carry, c.ph_cnt, c.ph_base, c.ph_tiles, c.ph_total, c.scal, c.red_ticket, c.bar64, c.err_word, c.stat_dev, c.inj_dev, c.inj_count,
+                    c.patch_coef, c.patch_coeff, c.red, c.coop_partial, c.rowkind, c.pcg_x, c.ph_tets, c.ph_Q, c.ph_carry, c.ph_cnt, c.ph_base, c.ph_tiles, c.ph_total, c.scal, c.red_ticket, c.bar64, c.err_word, c.inj_dev, c.inj_count,
                     c.inj_base, c.inj_carry, c.next_id};
     for (void* p : ptrs) lib_free(p);
     if (c.stat_host) cudaFreeHost(c.stat_host);
@@ -992,38 +991,29 @@ pifepic_status pifepic_set_external_E(pifepic_ctx* ctx, const double* E, int mem
     return PIFEPIC_OK;
 }
 
-static pifepic_status fill_stats(pifepic_ctx* ctx, const unsigned long long* before, pifepic_stats* st,
-                                 const float* phase_ms, long long it0, long long l0, long long nsolves,
-                                 long long ot0);
+// the statistics of a call from the context's two packs (after it and before it)
+static pifepic_status fill_stats(pifepic_ctx* ctx, pifepic_stats* st, const float* phase_ms, long long l0,
+                                 long long nsolves);
 
 }  // extern "C"
 
 namespace pf {
-// counters before a batched call, and the statistics after it (batch.cu)
-void snapshot_counters(pifepic_ctx* ctx, unsigned long long* before, long long* it0, long long* ot0, long long* l0) {
-    StatPack pk;
-    if (gather_stats(ctx->c, &pk, false) != cudaSuccess) memset(&pk, 0, sizeof(pk));
-    memcpy(before, pk.ctr, sizeof(pk.ctr));
-    *it0 = pk.it_total;
-    *ot0 = pk.outer_total;
-    *l0 = ctx->c.launches;
-}
-pifepic_status finish_stats(pifepic_ctx* ctx, const unsigned long long* before, long long it0, long long ot0,
-                            long long nsteps, long long kernels, pifepic_stats* st) {
-    long long l0 = ctx->c.launches - kernels;
-    return fill_stats(ctx, before, st, nullptr, it0, l0, 0, ot0);
+// a batch member's (batch.cu)
+pifepic_status finish_stats(pifepic_ctx* ctx, long long kernels, pifepic_stats* st) {
+    return fill_stats(ctx, st, nullptr, ctx->c.launches - kernels, 0);
 }
 }  // namespace pf
 
 extern "C" {
 
-static pifepic_status fill_stats(pifepic_ctx* ctx, const unsigned long long* before, pifepic_stats* st,
-                                 const float* phase_ms, long long it0, long long l0, long long nsolves,
-                                 long long ot0) {
+static pifepic_status fill_stats(pifepic_ctx* ctx, pifepic_stats* st, const float* phase_ms, long long l0,
+                                 long long nsolves) {
     Ctx& c = ctx->c;
-    StatPack pk;
-    cudaError_t e = gather_stats(c, &pk, c.have_object);
-    if (e != cudaSuccess) FAIL(PIFEPIC_ECUDA, "statistics: %s", cudaGetErrorString(e));
+    const StatPack &pk = c.stat_host[0], &pk0 = c.stat_host[1];
+    const unsigned long long* before = pk0.ctr;
+    c.last_iters = pk.it;
+    c.last_relres = pk.relres;
+    c.last_conv = pk.converged;
     const unsigned long long* now = pk.ctr;
     pifepic_stats s;
     memset(&s, 0, sizeof(s));
@@ -1041,10 +1031,10 @@ static pifepic_status fill_stats(pifepic_ctx* ctx, const unsigned long long* bef
         s.dropped[q] = (int64_t)(a[C_DROPPED] - b[C_DROPPED]);
         s.count[q] = pk.count[q];
     }
-    s.pcg_iters_total = pk.it_total - it0;
+    s.pcg_iters_total = pk.it_total - pk0.it_total;
     // host-launched kernels + the solve graph's kernels (the PCG is one persistent launch)
     s.kernel_launches = (c.launches - l0) + nsolves * solve_graph_fixed_kernels(c);
-    s.pcg_outer_total = pk.outer_total - ot0;
+    s.pcg_outer_total = pk.outer_total - pk0.outer_total;
     s.pcg_iters = c.last_iters;
     s.pcg_relres = c.last_relres;
     s.pcg_converged = c.last_conv;
@@ -1117,14 +1107,15 @@ pifepic_status pifepic_solve(pifepic_ctx* ctx, pifepic_stats* st) {
     NEED(ctx);
     Ctx& c = ctx->c;
     if (!c.have_object) FAIL(PIFEPIC_ESTATE, "set_object first");
-    unsigned long long before[MAX_SPECIES * NCTR];
-    long long it0, l0, ot0;
-    snapshot_counters(ctx, before, &it0, &ot0, &l0);
+    const long long l0 = c.launches;
+    Ctx* const cp = &c;
+    CUDA_OK(mark_stats(&cp, 1, c.stream));
     if (c.precision == PIFEPIC_MIXED) CUDA_OK(launch_deposit_all_mixed(c));
     else CUDA_OK(launch_deposit_all(c));
     if (!c.external_E) CUDA_OK(run_solve(c));
+    CUDA_OK(queue_stats(&cp, 1, c.stream));
     CUDA_OK(cudaStreamSynchronize(c.stream));
-    pifepic_status r = fill_stats(ctx, before, st, nullptr, it0, l0, c.external_E ? 0 : 1, ot0);
+    pifepic_status r = fill_stats(ctx, st, nullptr, l0, c.external_E ? 0 : 1);
     if (r || c.external_E) return r;
     c.solves_done += 1;
     return settle_solver(ctx);
@@ -1144,9 +1135,9 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
     Ctx& c = ctx->c;
     if (!c.have_object) FAIL(PIFEPIC_ESTATE, "set_object first");
     if (nsteps < 0) FAIL(PIFEPIC_EINVAL, "nsteps < 0");
-    unsigned long long before[MAX_SPECIES * NCTR];
-    long long it0, l0, ot0;
-    snapshot_counters(ctx, before, &it0, &ot0, &l0);
+    const long long l0 = c.launches;
+    Ctx* const cp = &c;
+    CUDA_OK(mark_stats(&cp, 1, c.stream));
     float ph[8] = {0};
     bool mixed = c.precision == PIFEPIC_MIXED;
     // The host does not wait for each step: every step records its six phase
@@ -1238,6 +1229,9 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
             if (g) return g;
         }
     }
+    // the statistics are queued behind the steps before the host waits for
+    // them; after the wait where a full waiting list may still be rebuilt
+    if (!each) CUDA_OK(queue_stats(&cp, 1, c.stream));
     for (int k = 0; k < STEP_RING; ++k) {   // the sets not read yet, oldest first
         const int slot = (nsteps + k) % STEP_RING;
         if (unread[slot]) CUDA_OK(read_set(slot));
@@ -1246,7 +1240,9 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
         pifepic_status g = check_spill((nsteps - 1) % STEP_RING);
         if (g) return g;
     }
-    pifepic_status r = fill_stats(ctx, before, st, ph, it0, l0, c.external_E ? 0 : nsteps, ot0);
+    if (each) CUDA_OK(queue_stats(&cp, 1, c.stream));
+    CUDA_OK(cudaStreamSynchronize(c.stream));
+    pifepic_status r = fill_stats(ctx, st, ph, l0, c.external_E ? 0 : nsteps);
     if (r || c.external_E || nsteps == 0) return r;
     c.solves_done += nsteps;
     return settle_solver(ctx);

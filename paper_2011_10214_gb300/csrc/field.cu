@@ -32,14 +32,6 @@ __constant__ TetTables cTf;
 __constant__ float cFold[2][81];
 
 // ---- right-hand side ----------------------------------------------------------
-struct RhsArgs {
-    const unsigned long long* W;     // [MAX_SPECIES][nnodes]
-    const unsigned long long* surf;  // [MAX_SPECIES][ncut]
-    const double* coefs;             // [MAX_SPECIES] q_s w_s (device)
-    const int* nspec;                // device
-    long long ncut;
-};
-
 __global__ void k_qcut(RhsArgs a, const double* area, double* qcut) {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (c >= a.ncut) return;
@@ -268,40 +260,6 @@ static void launch_node_E_f(const Ctx& c, cudaStream_t st) {
 }
 
 
-// ---- surface diagnostics: total collected charge, area-mean potential on Gamma_h ----
-__global__ void k_surface_diag(Mesh m, long long nit, const int* it_cell, const int* it_t, const double* it_data,
-                               const double* qT, const double* phi, double* partial, unsigned* ticket,
-                               double* out) {
-    long long T = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double v[2] = {0, 0};
-    // the object's surface only: a bedrock-plane tet lies inside the object
-    if (T < nit && it_data[T * IT_STRIDE + IT_KIND] == 0.0) {
-        const double* rec = it_data + T * IT_STRIDE;
-        int c = it_cell[T], t = it_t[T];
-        int i = c % m.nx, j = (c / m.nx) % m.ny, k = c / (m.nx * m.ny);
-        int p = (i + j + k) & 1;
-        double s = qT[T] * rec[IT_SJ];
-        for (int a = 0; a < 4; ++a) {
-            int av, bv, cv; loff(cTf.vert[p][t][a], av, bv, cv);
-            s += phi[node_id(m, i + av, j + bv, k + cv)] * rec[IT_S + a];
-        }
-        v[0] = s; v[1] = rec[IT_AREA];
-    }
-    double tot[2];
-    if (grid_sum<2>(v, partial, ticket, tot) && threadIdx.x == 0) out[0] = tot[1] > 0.0 ? tot[0] / tot[1] : 0.0;
-}
-
-__global__ void k_surface_charge(RhsArgs a, double* partial, unsigned* ticket, double* out) {
-    long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double v[1] = {0};
-    if (c < a.ncut) {
-        int ns = *a.nspec;
-        for (int s = 0; s < ns; ++s) v[0] += a.coefs[s] * (double)(long long)a.surf[(long long)s * a.ncut + c];
-    }
-    double tot[1];
-    if (grid_sum<1>(v, partial, ticket, tot) && threadIdx.x == 0) out[0] = tot[0];
-}
-
 // ------------------------------------------------------------------------------------
 static unsigned nb(long long n) { return (unsigned)((n + 255) / 256); }
 // device count of solves (PCG start extrapolation), scalar slot 43
@@ -327,7 +285,6 @@ static FieldArgs fargs(Ctx& c) {
 static PcgState* pcg_state(Ctx& c) { return (PcgState*)c.scal; }
 static double* coefs_dev(Ctx& c) { return c.scal + 16; }
 static int* nspec_dev(Ctx& c) { return (int*)(c.scal + 24); }
-static double* diag_dev(Ctx& c) { return c.scal + 32; }
 
 static RhsArgs rargs(Ctx& c) {
     RhsArgs a;
@@ -497,67 +454,95 @@ cudaError_t launch_solve_external(Ctx& c, const double* Fdev, int* iters, double
     return e;
 }
 
-struct StatArgs {
-    const unsigned long long* ctrall;
-    const int* bcount[MAX_SPECIES];
-    const unsigned long long* mov_n[MAX_SPECIES];
-    int nspecies, nblocks;
-    const double* scal;
-    const double* diag;   // surface charge, potential; null: not gathered
-    const int* err;
-    StatPack* out;
-};
+// ---- statistics of a call -------------------------------------------------------
+constexpr int ST_THREADS = 256, ST_BLOCKS = 304;   // (two blocks per SM; bounds the partials in c.red)
 
-// one block of 256 threads
-__global__ void k_stat_pack(StatArgs a) {
-    __shared__ long long part[8];
+// The packs are written straight into the contexts' pinned host blocks (some
+// 700 bytes, by one block at its end): no copy to queue, and the host waits for
+// the stream once per call.  The kernels take up to STAT_GROUP contexts.
+struct StatGroup {
+    StatArgs a[STAT_GROUP];
+};
+static_assert(sizeof(StatGroup) <= 4096, "kernel parameters");
+
+// the counters before the call's first step, one block per context
+__global__ void k_stat_mark(const __grid_constant__ StatGroup g) {
+    const StatArgs& a = g.a[blockIdx.x];
     const int t = threadIdx.x;
-    for (int i = t; i < MAX_SPECIES * NCTR; i += blockDim.x) a.out->ctr[i] = a.ctrall[i];
-    if (t < MAX_SPECIES) a.out->count[t] = 0;
-    for (int s = 0; s < a.nspecies && s < MAX_SPECIES; ++s) {   // (a.nspecies is the same in every thread)
-        long long v = 0;
-        if (a.bcount[s])
-            for (int b = t; b < a.nblocks; b += blockDim.x) v += a.bcount[s][b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((t & 31) == 0) part[t >> 5] = v;
-        __syncthreads();
-        if (t == 0) {
-            long long tot = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
-            if (a.mov_n[s]) tot += (long long)a.mov_n[s][0];
-            a.out->count[s] = tot;
-        }
-        __syncthreads();
-    }
+    if (t < MAX_SPECIES * NCTR) a.out[1].ctr[t] = a.ctrall[t];
     if (t == 0) {
-        const PcgState* S = (const PcgState*)a.scal;
-        a.out->it = S->it;
-        a.out->converged = S->converged;
-        a.out->relres = S->relres;
-        a.out->it_total = ((const long long*)a.scal)[40];
-        a.out->outer_total = ((const long long*)a.scal)[41];
-        a.out->surface_charge = a.diag ? a.diag[0] : 0.0;
-        a.out->surface_potential = a.diag ? a.diag[1] : 0.0;
-        a.out->err = *a.err;
+        a.out[1].it_total = ((const long long*)a.scal)[40];
+        a.out[1].outer_total = ((const long long*)a.scal)[41];
     }
 }
 
-cudaError_t gather_stats(Ctx& c, StatPack* out, bool diag) {
-    double* d = diag_dev(c);
-    if (diag) {
-        RhsArgs ra = rargs(c);
-        if (c.nit > 0)
-            k_surface_diag<<<nb(c.nit), 256, 0, c.stream>>>(c.mesh, c.nit, c.it_cell, c.it_t, c.it_data, c.qT, c.phi,
-                                                            c.red, c.red_ticket, d + 1);
-        else
-            cudaMemsetAsync(d + 1, 0, sizeof(double), c.stream);
-        if (c.ncut > 0)
-            k_surface_charge<<<nb(c.ncut), 256, 0, c.stream>>>(ra, c.red, c.red_ticket, d);
-        else
-            cudaMemsetAsync(d, 0, sizeof(double), c.stream);
+// After it, gridDim.y contexts: the object's area-mean potential on Gamma_h and
+// its collected charge, the species' particle counts, the solver's state.  One
+// pass over the interface tets, the cut cells and the bins, block partials, and
+// the last block to arrive packs the result: 5-9 us in one launch, where two
+// reductions and a one-block count were three launches of 5-10 us each (the
+// count alone 64-169 us with 250,000 bins).  Particle counts are summed in FP64
+// with the rest (exact below 2^53).
+__global__ void k_stat_pack(const __grid_constant__ StatGroup g) {
+    const StatArgs& a = g.a[blockIdx.y];
+    constexpr int NV = 3 + MAX_SPECIES;
+    double v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = 0.0;
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, dt = (long long)gridDim.x * blockDim.x;
+    const int ns = a.nspecies < MAX_SPECIES ? a.nspecies : MAX_SPECIES;
+    if (a.diag) {
+        const Mesh& m = a.m;
+        for (long long T = t0; T < a.nit; T += dt) {
+            // the object's surface only: a bedrock-plane tet lies inside the object
+            const double* rec = a.it_data + T * IT_STRIDE;
+            if (rec[IT_KIND] != 0.0) continue;
+            int c = a.it_cell[T], t = a.it_t[T];
+            int i = c % m.nx, j = (c / m.nx) % m.ny, k = c / (m.nx * m.ny);
+            int p = (i + j + k) & 1;
+            double s = a.qT[T] * rec[IT_SJ];
+            for (int q = 0; q < 4; ++q) {
+                int av, bv, cv; loff(cTf.vert[p][t][q], av, bv, cv);
+                s += a.phi[node_id(m, i + av, j + bv, k + cv)] * rec[IT_S + q];
+            }
+            v[0] += s; v[1] += rec[IT_AREA];
+        }
+        for (long long c = t0; c < a.rhs.ncut; c += dt) {
+            const int nsp = *a.rhs.nspec;
+            for (int s = 0; s < nsp; ++s)
+                v[2] += a.rhs.coefs[s] * (double)(long long)a.rhs.surf[(long long)s * a.rhs.ncut + c];
+        }
     }
+#pragma unroll
+    for (int s = 0; s < MAX_SPECIES; ++s)
+        if (s < ns && a.bcount[s])
+            for (long long b = t0; b < a.nblocks; b += dt) v[3 + s] += (double)a.bcount[s][b];
+    double tot[NV];
+    if (!grid_sum<NV>(v, a.partial, a.ticket, tot)) return;
+    StatPack* out = a.out;
+    if (threadIdx.x < MAX_SPECIES * NCTR) out->ctr[threadIdx.x] = a.ctrall[threadIdx.x];
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int s = 0; s < MAX_SPECIES; ++s)
+            out->count[s] = (long long)tot[3 + s] + (s < ns && a.mov_n[s] ? (long long)a.mov_n[s][0] : 0);
+        const PcgState* S = (const PcgState*)a.scal;
+        out->it = S->it;
+        out->converged = S->converged;
+        out->relres = S->relres;
+        out->it_total = ((const long long*)a.scal)[40];
+        out->outer_total = ((const long long*)a.scal)[41];
+        out->surface_charge = tot[2];
+        out->surface_potential = tot[1] > 0.0 ? tot[0] / tot[1] : 0.0;
+        out->err = *a.err;
+    }
+}
+
+static StatArgs stat_args(Ctx& c, bool diag) {
     StatArgs a = {};
+    a.m = c.mesh;
+    a.diag = diag;
+    a.nit = c.nit; a.it_cell = c.it_cell; a.it_t = c.it_t; a.it_data = c.it_data; a.qT = c.qT; a.phi = c.phi;
+    a.rhs = rargs(c);
     a.ctrall = c.ctrall;
     a.nspecies = (int)c.sp.size();
     for (int s = 0; s < a.nspecies && s < MAX_SPECIES; ++s) {
@@ -566,19 +551,38 @@ cudaError_t gather_stats(Ctx& c, StatPack* out, bool diag) {
     }
     a.nblocks = c.nblocks;
     a.scal = c.scal;
-    a.diag = diag ? d : nullptr;
     a.err = c.err_word;
-    a.out = c.stat_dev;
-    k_stat_pack<<<1, 256, 0, c.stream>>>(a);
-    cudaError_t e = cudaMemcpyAsync(c.stat_host, c.stat_dev, sizeof(StatPack), cudaMemcpyDeviceToHost, c.stream);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamSynchronize(c.stream);
-    if (e != cudaSuccess) return e;
-    *out = *c.stat_host;
-    c.last_iters = out->it;
-    c.last_relres = out->relres;
-    c.last_conv = out->converged;
-    return cudaSuccess;
+    a.partial = c.red;
+    a.ticket = c.red_ticket;
+    a.out = c.stat_host;
+    long long work = c.nblocks;
+    if (diag) work = std::max(work, std::max(c.nit, c.ncut));
+    a.blocks = (int)std::max(1ll, std::min((long long)ST_BLOCKS, (work + ST_THREADS - 1) / ST_THREADS));
+    return a;
+}
+
+cudaError_t mark_stats(Ctx* const* c, int n, cudaStream_t st) {
+    for (int i = 0; i < n; i += STAT_GROUP) {
+        StatGroup g = {};
+        const int k = std::min(STAT_GROUP, n - i);
+        for (int q = 0; q < k; ++q) g.a[q] = stat_args(*c[i + q], false);
+        k_stat_mark<<<k, MAX_SPECIES * NCTR, 0, st>>>(g);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t queue_stats(Ctx* const* c, int n, cudaStream_t st) {
+    for (int i = 0; i < n; i += STAT_GROUP) {
+        StatGroup g = {};
+        const int k = std::min(STAT_GROUP, n - i);
+        int blocks = 1;   // (a context with less work than the largest: its last blocks find none)
+        for (int q = 0; q < k; ++q) {
+            g.a[q] = stat_args(*c[i + q], c[i + q]->have_object);
+            blocks = std::max(blocks, g.a[q].blocks);
+        }
+        k_stat_pack<<<dim3(blocks, k), ST_THREADS, 0, st>>>(g);
+    }
+    return cudaGetLastError();
 }
 
 // FP64 node field from the current phi into E only (the FP32 copy the MIXED

@@ -180,6 +180,36 @@ struct StatPack {
     int it, converged, err, pad;
 };
 
+// the right-hand side's particle charges
+struct RhsArgs {
+    const unsigned long long* W;     // [MAX_SPECIES][nnodes]
+    const unsigned long long* surf;  // [MAX_SPECIES][ncut]
+    const double* coefs;             // [MAX_SPECIES] q_s w_s (device)
+    const int* nspec;                // device
+    long long ncut;
+};
+
+// what the statistics of one context read, and where they go: out[0] after the
+// call, out[1] the counters before it
+constexpr int STAT_GROUP = 8;
+struct StatArgs {
+    Mesh m;
+    long long nit;
+    const int *it_cell, *it_t;
+    const double *it_data, *qT, *phi;
+    RhsArgs rhs;
+    const unsigned long long* ctrall;
+    const int* bcount[MAX_SPECIES];
+    const unsigned long long* mov_n[MAX_SPECIES];
+    int nspecies, nblocks, blocks;
+    bool diag;            // the surface charge and potential are gathered too
+    const double* scal;
+    const int* err;
+    double* partial;      // [3 + MAX_SPECIES][blocks]
+    unsigned* ticket;
+    StatPack* out;
+};
+
 struct Ctx {
     std::string err;
     cudaStream_t stream = nullptr;
@@ -300,8 +330,7 @@ struct Ctx {
     long long pcg_M = 0;
     size_t pcg_smem = 0;
     int* err_word = nullptr;
-    StatPack* stat_dev = nullptr;   // gather_stats: device block and its pinned host copy
-    StatPack* stat_host = nullptr;
+    StatPack* stat_host = nullptr;  // statistics after a call and before it (pinned, written by the device)
     // graphs
     cudaGraphExec_t pcg_exec = nullptr;
     cudaGraph_t pcg_graph = nullptr;
@@ -390,7 +419,11 @@ cudaError_t build_pcg_graph(Ctx& c);                   // field.cu
 void plan_pcg(Ctx& c);                                 // pcg_coop.cu
 cudaError_t launch_pcg(Ctx& c);
 // diag: also the surface charge and mean surface potential (a few kernels)
-cudaError_t gather_stats(Ctx& c, StatPack* out, bool diag);
+// statistics of a call over n contexts: mark_stats queues the reading of the
+// counters before it, queue_stats the gathering after it, into each context's
+// stat_host[1] and [0]; both are there once st has been waited for
+cudaError_t mark_stats(Ctx* const* c, int n, cudaStream_t st);
+cudaError_t queue_stats(Ctx* const* c, int n, cudaStream_t st);
 cudaError_t launch_qtets(Ctx& c);
 
 Launch make_launch(Ctx& c);
