@@ -113,78 +113,125 @@ __global__ void k_u_from_phi(long long N, const int* ntype, const double* phi, d
 }
 
 // ---- node field ---------------------------------------------------------------------
-__global__ void k_node_E(FieldArgs f, const double* L, const unsigned char* imask, const int* ibase,
-                         const double* it_data, const double* qT, const double* phi, double4* E, float4* Ef) {
+// Minus the volume-weighted mean of the element gradients around a node, the
+// plasma-side pieces if there are any.  A block takes 4 x 4 x 4 nodes: first each
+// tet of its 5 x 5 x 5 cells once, into shared memory (its volume times gradient
+// and its volume, plasma side and whole), then each node's eight sums over its 8
+// or 32 tets, in cell order, one sum per thread (a warp takes nodes of one parity,
+// which have the same tets).  FP64-bound: about 310 operations a node, where a
+// thread per node spent 770 on its 20 tets and the interface's nodes in turn
+// made one thread the tail.  16^3 cells: 107 -> 23 us, 40^3: 219 -> 75.
+constexpr int N64_T = 4, N64_C = N64_T + 1, N64_TETS = N64_C * N64_C * N64_C * 5, N64_GRAD = 13;
+__global__ void __launch_bounds__(256) k_node_E(FieldArgs f, const double* L, const unsigned char* imask, const int* ibase,
+                                                const double* it_data, const double* qT, const double* phi, double4* E,
+                                                float4* Ef) {
+    enum { APL = 0, VPL = 3, AAL = 4, VAL = 7 };
+    __shared__ double ct[8][N64_TETS];
+    __shared__ double res[8][N64_T * N64_T * N64_T];
+    __shared__ double grad[2 * 5 * N64_GRAD], vol[5], s_ih;
+    __shared__ int vert[2 * 5 * 4], has[2 * 8];   // has: the tets of a cell of parity p at its corner c8, as bits
     const Mesh& m = f.m;
-    long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= m.nnodes) return;
-    int i, j, k;
-    node_ijk(m, n, i, j, k);
-    double apl[3] = {0, 0, 0}, vpl = 0.0, aal[3] = {0, 0, 0}, val = 0.0;
-    double ih = 1.0 / m.h, V3 = m.h * m.h * m.h;
-    for (int c8 = 0; c8 < 8; ++c8) {
-        int a, b, c; loff(c8, a, b, c);
-        int ci = i - a, cj = j - b, ck = k - c;
-        if (ci < 0 || cj < 0 || ck < 0 || ci >= m.nx || cj >= m.ny || ck >= m.nz) continue;
-        long long cell = cell_id(m, ci, cj, ck);
-        unsigned mk = imask[cell];
-        int p = (ci + cj + ck) & 1;
-        int T = ibase[cell];
-        for (int t = 0; t < 5; ++t) {
-            bool itet = (mk >> t) & 1;
-            bool has = false;
+    const int tid = threadIdx.x;
+    const int i0 = blockIdx.x * N64_T, j0 = blockIdx.y * N64_T, k0 = blockIdx.z * N64_T;
+    if (tid < 120) grad[(tid / 12) * N64_GRAD + tid % 12] = (&cTf.grad[0][0][0][0])[tid];
+    else if (tid >= 128 && tid < 133) vol[tid - 128] = cTf.vol[tid - 128];
+    else if (tid >= 160 && tid < 200) vert[tid - 160] = (&cTf.vert[0][0][0])[tid - 160];
+    else if (tid >= 224 && tid < 240) {
+        int bits = 0;
+        for (int t = 0; t < 5; ++t)
             for (int v = 0; v < 4; ++v)
-                if (cTf.vert[p][t][v] == c8) has = true;
-            if (has) {
-                double ph[4];
-                long long nd0 = 0;
-                for (int v = 0; v < 4; ++v) {
-                    int av, bv, cv; loff(cTf.vert[p][t][v], av, bv, cv);
-                    long long nd = node_id(m, ci + av, cj + bv, ck + cv);
-                    if (v == 0) nd0 = nd;
-                    ph[v] = phi[nd];
-                }
-                if (itet) {
-                    const double* rec = it_data + (long long)T * IT_STRIDE;
-                    double qt = qT[T];
-                    double gp[3], gm[3];
-                    for (int d = 0; d < 3; ++d) {
-                        gp[d] = ph[0] * rec[IT_GP + d] + ph[1] * rec[IT_GP + 3 + d] + ph[2] * rec[IT_GP + 6 + d] +
-                                ph[3] * rec[IT_GP + 9 + d] + qt * rec[IT_GP + 12 + d];
-                        gm[d] = ph[0] * rec[IT_GM + d] + ph[1] * rec[IT_GM + 3 + d] + ph[2] * rec[IT_GM + 6 + d] +
-                                ph[3] * rec[IT_GM + 9 + d] + qt * rec[IT_GM + 12 + d];
-                    }
-                    double vp = rec[IT_VOLP], vm = rec[IT_VOLM];
-                    // the + piece is plasma on the object's surface only (not on the bedrock plane)
-                    if (vp > 0.0 && rec[IT_KIND] == 0.0) {
-                        for (int d = 0; d < 3; ++d) apl[d] += vp * gp[d];
-                        vpl += vp;
-                    }
-                    for (int d = 0; d < 3; ++d) aal[d] += vp * gp[d] + vm * gm[d];
-                    val += vp + vm;
-                } else {
-                    double g[3];
-                    for (int d = 0; d < 3; ++d)
-                        g[d] = (ph[0] * cTf.grad[p][t][0][d] + ph[1] * cTf.grad[p][t][1][d] +
-                                ph[2] * cTf.grad[p][t][2][d] + ph[3] * cTf.grad[p][t][3][d]) * ih;
-                    double V = cTf.vol[t] * V3;
-                    if (L[nd0] >= 0.0) {
-                        for (int d = 0; d < 3; ++d) apl[d] += V * g[d];
-                        vpl += V;
-                    }
-                    for (int d = 0; d < 3; ++d) aal[d] += V * g[d];
-                    val += V;
-                }
-            }
-            if (itet) ++T;
-        }
+                if (cTf.vert[(tid - 224) >> 3][t][v] == (tid & 7)) bits |= 1 << t;
+        has[tid - 224] = bits;
+    } else if (tid == 255) {
+        s_ih = 1.0 / m.h;   // (once: an FP64 division is some ten instructions)
     }
+    __syncthreads();
+    const double ih = s_ih, V3 = m.h * m.h * m.h;
+    for (int q = tid; q < N64_TETS; q += 256) {
+        const int t = q % 5, cell = q / 5;
+        const int ci = i0 - 1 + cell % N64_C, cj = j0 - 1 + cell / N64_C % N64_C, ck = k0 - 1 + cell / (N64_C * N64_C);
+        if (ci < 0 || cj < 0 || ck < 0 || ci >= m.nx || cj >= m.ny || ck >= m.nz) continue;
+        const long long id = cell_id(m, ci, cj, ck);
+        const unsigned mk = imask[id];
+        const int tet = ((ci + cj + ck) & 1) * 5 + t;
+        double ph[4];
+        long long nd0 = 0;
+        for (int v = 0; v < 4; ++v) {
+            int av, bv, cv; loff(vert[tet * 4 + v], av, bv, cv);
+            const long long nd = node_id(m, ci + av, cj + bv, ck + cv);
+            if (v == 0) nd0 = nd;
+            ph[v] = phi[nd];
+        }
+        double o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if ((mk >> t) & 1) {
+            const int T = ibase[id] + __popc(mk & ((1u << t) - 1));
+            const double* rec = it_data + (long long)T * IT_STRIDE;
+            const double qt = qT[T], vp = rec[IT_VOLP], vm = rec[IT_VOLM];
+            // the + piece is plasma on the object's surface only (not on the bedrock plane)
+            const bool plasma = vp > 0.0 && rec[IT_KIND] == 0.0;
+            for (int d = 0; d < 3; ++d) {
+                const double gp = ph[0] * rec[IT_GP + d] + ph[1] * rec[IT_GP + 3 + d] + ph[2] * rec[IT_GP + 6 + d] +
+                                  ph[3] * rec[IT_GP + 9 + d] + qt * rec[IT_GP + 12 + d];
+                const double gm = ph[0] * rec[IT_GM + d] + ph[1] * rec[IT_GM + 3 + d] + ph[2] * rec[IT_GM + 6 + d] +
+                                  ph[3] * rec[IT_GM + 9 + d] + qt * rec[IT_GM + 12 + d];
+                if (plasma) o[APL + d] = vp * gp;
+                o[AAL + d] = vp * gp + vm * gm;
+            }
+            if (plasma) o[VPL] = vp;
+            o[VAL] = vp + vm;
+        } else {
+            const double* gr = grad + tet * N64_GRAD;
+            const double V = vol[t] * V3;
+            const bool plasma = L[nd0] >= 0.0;
+            for (int d = 0; d < 3; ++d) {
+                const double g = (ph[0] * gr[d] + ph[1] * gr[3 + d] + ph[2] * gr[6 + d] + ph[3] * gr[9 + d]) * ih;
+                o[AAL + d] = V * g;
+                if (plasma) o[APL + d] = V * g;
+            }
+            if (plasma) o[VPL] = V;
+            o[VAL] = V;
+        }
+#pragma unroll
+        for (int d = 0; d < 8; ++d) ct[d][q] = o[d];
+    }
+    __syncthreads();
+    for (int half = 0; half < 2; ++half) {
+        const int lane = tid & 31, odd = (tid >> 5) & 1, d = 4 * half + (tid >> 6);   // (a warp: one sum of the 32 nodes of a parity)
+        const int z = lane >> 3, y = (lane >> 1) & 3, x = 2 * (lane & 1) + ((odd + y + z + i0 + j0 + k0) & 1);
+        const int i = i0 + x, j = j0 + y, k = k0 + z;
+        double sum = 0.0;
+        // (the sums over all pieces only where there is no plasma)
+        if (i <= m.nx && j <= m.ny && k <= m.nz && !(half && res[VPL][x + N64_T * (y + N64_T * z)] > 0.0))
+            for (int c8 = 0; c8 < 8; ++c8) {
+                int a, b, c; loff(c8, a, b, c);
+                const int ci = i - a, cj = j - b, ck = k - c;
+                if (ci < 0 || cj < 0 || ck < 0 || ci >= m.nx || cj >= m.ny || ck >= m.nz) continue;
+                const double* tets = ct[d] + 5 * ((x + 1 - a) + N64_C * ((y + 1 - b) + N64_C * (z + 1 - c)));
+                const int bits = has[((ci + cj + ck) & 1) * 8 + c8];
+                for (int t = 0; t < 5; ++t)
+                    if ((bits >> t) & 1) sum += tets[t];
+            }
+        res[d][x + N64_T * (y + N64_T * z)] = sum;
+        __syncthreads();
+    }
+    if (tid >= N64_T * N64_T * N64_T) return;
+    const int i = i0 + tid % N64_T, j = j0 + tid / N64_T % N64_T, k = k0 + tid / (N64_T * N64_T);
+    if (i > m.nx || j > m.ny || k > m.nz) return;
+    const bool plasma = res[VPL][tid] > 0.0;
+    const int g = plasma ? APL : AAL;
+    const double w = res[plasma ? VPL : VAL][tid];
     double4 e;
-    if (vpl > 0.0) { e.x = -apl[0] / vpl; e.y = -apl[1] / vpl; e.z = -apl[2] / vpl; }
-    else { e.x = -aal[0] / val; e.y = -aal[1] / val; e.z = -aal[2] / val; }
+    e.x = -res[g][tid] / w; e.y = -res[g + 1][tid] / w; e.z = -res[g + 2][tid] / w;
     e.w = 0.0;
+    const long long n = node_id(m, i, j, k);
     E[n] = e;
     if (Ef) Ef[n] = make_float4((float)e.x, (float)e.y, (float)e.z, 0.0f);
+}
+
+static void launch_node_E(const FieldArgs& f, const Ctx& c, float4* Ef, cudaStream_t st) {
+    const Mesh& m = c.mesh;
+    const dim3 grid((m.NX + N64_T - 1) / N64_T, (m.NY + N64_T - 1) / N64_T, (m.NZ + N64_T - 1) / N64_T);
+    k_node_E<<<grid, 256, 0, st>>>(f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi, c.E, Ef);
 }
 
 // Node field in FP32 (MIXED steps; the push reads only this copy).  Same
@@ -351,8 +398,7 @@ static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     e = fd ? launch_pcg_fd(c, st) : launch_pcg_coop(c, st);
     if (e != cudaSuccess) return e;
     if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, st);
-    else k_node_E<<<node_blocks(N), node_threads(N), 0, st>>>(f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi,
-                                                               c.E, c.Ef);
+    else launch_node_E(f, c, c.Ef, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_E_to_pic(c, st, c.precision != PIFEPIC_MIXED);
@@ -373,8 +419,7 @@ cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st, bool fd) {
 cudaError_t launch_solve_suffix(Ctx& c, cudaStream_t st) {
     FieldArgs f = fargs(c);
     if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, st);
-    else k_node_E<<<node_blocks(c.mesh.nnodes), node_threads(c.mesh.nnodes), 0, st>>>(
-        f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi, c.E, c.Ef);
+    else launch_node_E(f, c, c.Ef, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_E_to_pic(c, st, c.precision != PIFEPIC_MIXED);
@@ -470,6 +515,7 @@ __global__ void k_stat_mark(const __grid_constant__ StatGroup g) {
     const StatArgs& a = g.a[blockIdx.x];
     const int t = threadIdx.x;
     if (t < MAX_SPECIES * NCTR) a.out[1].ctr[t] = a.ctrall[t];
+    if (t < MAX_SPECIES) a.count[t] = 0ull;
     if (t == 0) {
         a.out[1].it_total = ((const long long*)a.scal)[40];
         a.out[1].outer_total = ((const long long*)a.scal)[41];
@@ -479,16 +525,13 @@ __global__ void k_stat_mark(const __grid_constant__ StatGroup g) {
 // After it, gridDim.y contexts: the object's area-mean potential on Gamma_h and
 // its collected charge, the species' particle counts, the solver's state.  One
 // pass over the interface tets, the cut cells and the bins, block partials, and
-// the last block to arrive packs the result: 5-9 us in one launch, where two
-// reductions and a one-block count were three launches of 5-10 us each (the
-// count alone 64-169 us with 250,000 bins).  Particle counts are summed in FP64
-// with the rest (exact below 2^53).
+// the last block to arrive packs the result.  The counts are integers (added
+// to cleared words): eight more FP64 sums made the launch 23-33 us, not 12-15.
+// Two reductions and a one-block count were three launches of 5-10 us each (the
+// count alone 64-169 us with 250,000 bins).
 __global__ void k_stat_pack(const __grid_constant__ StatGroup g) {
     const StatArgs& a = g.a[blockIdx.y];
-    constexpr int NV = 3 + MAX_SPECIES;
-    double v[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] = 0.0;
+    double v[3] = {0.0, 0.0, 0.0};
     const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, dt = (long long)gridDim.x * blockDim.x;
     const int ns = a.nspecies < MAX_SPECIES ? a.nspecies : MAX_SPECIES;
     if (a.diag) {
@@ -515,16 +558,22 @@ __global__ void k_stat_pack(const __grid_constant__ StatGroup g) {
     }
 #pragma unroll
     for (int s = 0; s < MAX_SPECIES; ++s)
-        if (s < ns && a.bcount[s])
-            for (long long b = t0; b < a.nblocks; b += dt) v[3 + s] += (double)a.bcount[s][b];
-    double tot[NV];
-    if (!grid_sum<NV>(v, a.partial, a.ticket, tot)) return;
+        if (s < ns && a.bcount[s]) {
+            // (a warp's sum stays below 2^32: 32 lanes, nblocks / dt bins each, BIN_MAX particles a bin)
+            unsigned n = 0;
+            for (long long b = t0; b < a.nblocks; b += dt) n += (unsigned)a.bcount[s][b];
+            n = __reduce_add_sync(0xffffffffu, n);
+            if ((threadIdx.x & 31) == 0 && n) atomicAdd(a.count + s, (unsigned long long)n);
+        }
+    double tot[3];
+    if (!grid_sum<3>(v, a.partial, a.ticket, tot)) return;   // (fences behind the counts too)
     StatPack* out = a.out;
+    if (threadIdx.x >= 128 && threadIdx.x < 128 + MAX_SPECIES) {
+        const int s = threadIdx.x - 128;
+        out->count[s] = (long long)__ldcg(a.count + s) + (s < ns && a.mov_n[s] ? (long long)a.mov_n[s][0] : 0);
+    }
     if (threadIdx.x < MAX_SPECIES * NCTR) out->ctr[threadIdx.x] = a.ctrall[threadIdx.x];
     if (threadIdx.x == 0) {
-#pragma unroll
-        for (int s = 0; s < MAX_SPECIES; ++s)
-            out->count[s] = (long long)tot[3 + s] + (s < ns && a.mov_n[s] ? (long long)a.mov_n[s][0] : 0);
         const PcgState* S = (const PcgState*)a.scal;
         out->it = S->it;
         out->converged = S->converged;
@@ -552,7 +601,8 @@ static StatArgs stat_args(Ctx& c, bool diag) {
     a.nblocks = c.nblocks;
     a.scal = c.scal;
     a.err = c.err_word;
-    a.partial = c.red;
+    a.count = (unsigned long long*)c.red;
+    a.partial = c.red + MAX_SPECIES;
     a.ticket = c.red_ticket;
     a.out = c.stat_host;
     long long work = c.nblocks;
@@ -588,9 +638,7 @@ cudaError_t queue_stats(Ctx* const* c, int n, cudaStream_t st) {
 // FP64 node field from the current phi into E only (the FP32 copy the MIXED
 // push reads is left as the step made it)
 cudaError_t launch_node_E64(Ctx& c) {
-    FieldArgs f = fargs(c);
-    k_node_E<<<node_blocks(c.mesh.nnodes), node_threads(c.mesh.nnodes), 0, c.stream>>>(
-        f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi, c.E, nullptr);
+    launch_node_E(fargs(c), c, nullptr, c.stream);
     return cudaGetLastError();
 }
 

@@ -148,12 +148,11 @@ static __device__ __forceinline__ T apply_row_ld(const FieldArgs& f, long long n
 // conversions (FP64 issues slowly on this part); any other row goes through
 // apply_row_ld
 template <typename LD>
-static __device__ __forceinline__ double apply_row64(const FieldArgs& f, long long n, int i, int j, int k, LD ld,
-                                                     const double* coef) {
+static __device__ __forceinline__ double apply_row64_ty(const FieldArgs& f, long long n, int i, int j, int k, int ty,
+                                                        LD ld, const double* coef) {
     const Mesh& m = f.m;
-    const int ty = f.ntype[n];
     if (ty >= 0 || ty == -3 || i == 0 || j == 0 || k == 0 || i == m.nx || j == m.ny || k == m.nz)
-        return apply_row_ld<double>(f, n, i, j, k, ld, coef);
+        return apply_row_ty<double>(f, n, i, j, k, ty, ld, coef);
     const long long sx = 1, sy = m.NX, sz = (long long)m.NX * m.NY;
     const double eps = ty == -2 ? f.o.eps_minus : f.o.eps_plus;
     const bool odd = (i + j + k) & 1;
@@ -167,6 +166,11 @@ static __device__ __forceinline__ double apply_row64(const FieldArgs& f, long lo
         y -= (2.0 * m.h12) * ((dxy + dxz) + dyz);
     }
     return eps * y;
+}
+template <typename LD>
+static __device__ __forceinline__ double apply_row64(const FieldArgs& f, long long n, int i, int j, int k, LD ld,
+                                                     const double* coef) {
+    return apply_row64_ty(f, n, i, j, k, f.ntype[n], ld, coef);
 }
 
 // Row kinds for the masked regular stencil: the six neighbour-presence flags,

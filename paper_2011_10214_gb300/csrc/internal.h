@@ -205,7 +205,8 @@ struct StatArgs {
     bool diag;            // the surface charge and potential are gathered too
     const double* scal;
     const int* err;
-    double* partial;      // [3 + MAX_SPECIES][blocks]
+    unsigned long long* count;   // [MAX_SPECIES] particles in the bins, cleared by the marking
+    double* partial;             // [3][blocks]
     unsigned* ticket;
     StatPack* out;
 };
@@ -329,6 +330,7 @@ struct Ctx {
     int pcg_G = 1;
     long long pcg_M = 0;
     size_t pcg_smem = 0;
+    int pcg_stage = 0;            // FP64: general rows a block keeps in shared memory
     int* err_word = nullptr;
     StatPack* stat_host = nullptr;  // statistics after a call and before it (pinned, written by the device)
     // graphs

@@ -20,6 +20,7 @@
 // global memory / L2 (larger meshes, e.g. 160 x 160 x 80).
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "field_common.cuh"
@@ -52,9 +53,9 @@ constexpr int PIPE_STALL = 40;
 // outer FP64 residual corrects what FP32 inner products lose).  An exchange
 // is a monotonic arrival counter (below) with the block partials in one of two
 // slots by exchange parity, so a block that races ahead into the next exchange
-// never overwrites partials a slower block is still summing; the FP32 inner
-// loop of MIXED mode uses the fixed-point exchange instead, which needs no
-// second round trip for the partials.  z alternates between two copies by
+// never overwrites partials a slower block is still summing; the iterations of
+// both modes use the fixed-point exchanges instead, which need no second round
+// trip for the partials.  z alternates between two copies by
 // iteration parity: the update writes the copy that the previous iteration's
 // staging read, whose readers the previous r.z exchange (release/acquire)
 // already ordered before the writer.  So the p.q exchange orders no global
@@ -66,6 +67,7 @@ constexpr int PIPE_STALL = 40;
 
 constexpr int REG_THREADS = 512;
 
+constexpr int ROW_STAGED = 1 << 29;
 struct RegArgs {
     FieldArgs f;
     const double* b;
@@ -74,11 +76,13 @@ struct RegArgs {
     double* phi;
     void* zg[2];               // exchanged vector z (T), two guarded copies
     long long M;               // nodes per block
+    int stage_rows, stage_at;  // FP64: general rows a block keeps in shared memory, at that byte
     int woff[19];              // staged rows: window offset of each stencil slot
     double* val;               // [2][4][G] block partials
     unsigned long long* arrivals;  // grows by G per exchange
     unsigned long long* fx;        // fixed-point exchange words: pq at [0], r.r and r.z at [FX_LINE], [2 FX_LINE];
-                                   // pipelined loop: two sets of three at [(3 + 3 set + q) FX_LINE]
+                                   // pipelined loop: two sets of three at [(3 + 3 set + q) FX_LINE];
+                                   // FP64: the pieces of pq at [c FX_LINE], of r.r and r.z at [(3 + 3 q + c) FX_LINE]
     int* classic;                  // MIXED: 1 once a solve found the pipelined recurrences too inexact
     const int* hold;               // arrivals the launch's first exchange waits for beyond the grid (tests)
     PcgState* S;
@@ -123,6 +127,13 @@ static __host__ __device__ __forceinline__ void z_window_padded(long long NX, lo
     we = (b1 + halo + VEC - 1) / VEC * VEC;
 }
 
+// a <= b for a sum of squares and a positive bound: FP64 by their bits (a
+// comparison by every warp of a block takes a quarter of a microsecond)
+static __device__ __forceinline__ bool le_bits(float a, float b) { return a <= b; }
+static __device__ __forceinline__ bool le_bits(double a, double b) {
+    return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+
 // Jacobi PCG, vectors in registers.  FP64 mode: one pass in FP64.  MIXED: FP64
 // refinement (true residual of u in FP64) around FP32 inner solves for x.
 // ROWS: the block's operator rows are built once into shared memory ([node][19]
@@ -138,6 +149,10 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
     const FieldArgs& f = a.f;
     const long long N = f.m.nnodes;
     const long long NXY = (long long)f.m.NX * f.m.NY;
+    double quot = 0.0;   // FP64: the last exchange's quotient, alpha or beta
+    // this thread's node of each 512: FP64 gives a warp every second one, whose
+    // rows are mostly of one parity (7 or 19 terms)
+    const int tn = MIXED ? (int)threadIdx.x : (int)(threadIdx.x & ~63u) + 2 * (int)(threadIdx.x & 31u) + (int)((threadIdx.x >> 5) & 1u);
     const long long b0 = (long long)blockIdx.x * a.M;
     const long long b1 = b0 + a.M < N ? b0 + a.M : N;
     const int nown = (int)(b1 - b0);
@@ -171,18 +186,36 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
         }
         // rows are read only after the first exchange's __syncthreads
     }
+    __shared__ int nstaged;
+    if (!MIXED) {
+        if (threadIdx.x == 0) nstaged = 0;
+        __syncthreads();
+    }
     unsigned pk[NPT];
+    int ty[NPT];      // FP64: the row's kind; a general row staged in shared memory: ROW_STAGED + its place there
     T dv[NPT];
 #pragma unroll
     for (int s = 0; s < NPT; ++s) {
-        const long long n = b0 + threadIdx.x + s * REG_THREADS;
+        const long long n = b0 + tn + s * REG_THREADS;
         pk[s] = 0;
+        ty[s] = -3;
         dv[s] = (T)0;
         if (n < b1) {
             int i, j, kk;
             node_ijk(f.m, n, i, j, kk);
             pk[s] = pack_ijk(i, j, kk);
             dv[s] = dinv[n];
+            if (!MIXED) {
+                ty[s] = f.ntype[n];
+                if (ty[s] >= 0) {
+                    const int at = atomicAdd(&nstaged, 1);
+                    if (at < a.stage_rows) {
+                        double* row = (double*)(win_raw + a.stage_at) + 19 * at;
+                        for (int q = 0; q < 19; ++q) row[q] = f.coef[(long long)ty[s] * 19 + q];
+                        ty[s] = ROW_STAGED + at;
+                    }
+                }
+            }
         }
     }
     // this launch's starting values of the fixed-point words (read before the
@@ -191,6 +224,10 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
     if (MIXED && threadIdx.x < 2) {
         fxa = ld_relaxed(a.fx);
         fxb = ld_relaxed(a.fx + (1 + threadIdx.x) * FX_LINE);
+    }
+    if (!MIXED && threadIdx.x < 6) {
+        if (threadIdx.x < 3) fxa = ld_relaxed(a.fx + threadIdx.x * FX_LINE);
+        fxb = ld_relaxed(a.fx + (3 + threadIdx.x) * FX_LINE);
     }
     // pipelined loop: two word sets used in turn (a set is reused only after an
     // exchange on the other one, so every block has read its last total);
@@ -227,7 +264,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
     // row n (slot s of this thread) of the operator times the staged window
     auto apply = [&](int s, long long n) -> T {
         if (ROWS) {
-            const int li = threadIdx.x + s * REG_THREADS;
+            const int li = tn + s * REG_THREADS;
             const T* rw = rows + li * 19;
             const T* wc = win + (n - ws);
             T az = rw[0] * wc[0];
@@ -235,7 +272,12 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
             for (int q = 1; q < 19; ++q) az += rw[q] * wc[a.woff[q]];
             return az;
         }
-        return row_at<T>(f, n, pk[s], ldw, coef);
+        if constexpr (MIXED) return row_at<T>(f, n, pk[s], ldw, coef);
+        else {
+            const bool st = ty[s] >= ROW_STAGED;
+            return apply_row64_ty(f, n, (int)(pk[s] & 2047u), (int)((pk[s] >> 11) & 2047u), (int)(pk[s] >> 22),
+                                  st ? ty[s] - ROW_STAGED : ty[s], ldw, st ? (const double*)(win_raw + a.stage_at) : coef);
+        }
     };
     int it = 0, outer = 0;
     double bb = 0.0, rr = 0.0;
@@ -247,7 +289,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
         double v3[3] = {0.0, 0.0, 0.0};
 #pragma unroll
         for (int s = 0; s < NPT; ++s) {
-            const long long n = b0 + threadIdx.x + s * REG_THREADS;
+            const long long n = b0 + tn + s * REG_THREADS;
             x[s] = r[s] = z[s] = p[s] = q[s] = (T)0;
             if (n < b1) {
                 const double bn = a.b[n];
@@ -293,7 +335,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
             stage(zbuf[zc]);
 #pragma unroll
             for (int s = 0; s < NPT; ++s) {
-                const long long n = b0 + threadIdx.x + s * REG_THREADS;
+                const long long n = b0 + tn + s * REG_THREADS;
                 w[s] = sv[s] = nz[s] = (T)0;
                 if (n < b1) w[s] = apply(s, n);
             }
@@ -310,7 +352,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
                 T v[3] = {(T)0, (T)0, (T)0};
 #pragma unroll
                 for (int s = 0; s < NPT; ++s) {
-                    const long long n = b0 + threadIdx.x + s * REG_THREADS;
+                    const long long n = b0 + tn + s * REG_THREADS;
                     if (n < b1) {
                         zbuf[zc ^ 1][n] = dv[s] * w[s];
                         v[0] += r[s] * z[s];
@@ -351,7 +393,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
                 stage(zbuf[zc]);
 #pragma unroll
                 for (int s = 0; s < NPT; ++s) {
-                    const long long n = b0 + threadIdx.x + s * REG_THREADS;
+                    const long long n = b0 + tn + s * REG_THREADS;
                     if (n < b1) {
                         const T nn = apply(s, n);
                         const T m = dv[s] * w[s];
@@ -379,7 +421,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
           }
         } else {
             T beta = (T)0;
-            float pq_prev = 0.0f;     // no scale for the first p.q of an inner solve
+            T pq_prev = (T)0;         // no scale for the first p.q of an inner solve
             bool first = true;
             for (;;) {
                 stage(zbuf[zc]);
@@ -388,7 +430,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
                 const T bt = beta;
 #pragma unroll
                 for (int s = 0; s < NPT; ++s) {
-                    const long long n = b0 + threadIdx.x + s * REG_THREADS;
+                    const long long n = b0 + tn + s * REG_THREADS;
                     if (n < b1) {
                         const T az = apply(s, n);
                         if (first) {
@@ -407,14 +449,17 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
                     alive = exchange_f32<1, false, 8>(a, e, a.fx, fxa, rf, fx_ref_ok(pq_prev), v1, pq, xs);
                     pq_prev = pq[0];
                 } else {
-                    alive = exchange<T, 1>(a, e, v1, pq, xs);
+                    const double rf[1] = {(double)pq_prev};
+                    alive = exchange_f64<1, false>(a, e, a.fx, fxa, rf, v1, pq,
+                                                   [=](const double (&t)[1]) { return rz / t[0]; }, quot, xs);
+                    pq_prev = pq[0];
                 }
                 if (!alive) break;
-                const T al = rz / pq[0];
+                const T al = MIXED ? rz / pq[0] : (T)quot;
                 T v2[2] = {(T)0, (T)0};
 #pragma unroll
                 for (int s = 0; s < NPT; ++s) {
-                    const long long n = b0 + threadIdx.x + s * REG_THREADS;
+                    const long long n = b0 + tn + s * REG_THREADS;
                     if (n < b1) {
                         x[s] = x[s] + al * p[s];
                         r[s] = r[s] - al * q[s];
@@ -430,15 +475,17 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
                     alive = exchange_f32<2, true, 8>(a, e, a.fx + FX_LINE, fxb, rf, fx_ref_ok(rr_in) && fx_ref_ok(rz),
                                                      v2, t2, xs);
                 } else {
-                    alive = exchange<T, 2>(a, e, v2, t2, xs);
+                    const double rf[2] = {(double)rr_in, (double)rz};
+                    alive = exchange_f64<2, true>(a, e, a.fx + 3 * FX_LINE, fxb, rf, v2, t2,
+                                                  [=](const double (&t)[2]) { return t[1] / rz; }, quot, xs);
                 }
                 if (!alive) break;
                 zc ^= 1;
-                beta = t2[1] / rz;
+                beta = MIXED ? t2[1] / rz : (T)quot;
                 rz = t2[1];
                 rr_in = t2[0];
                 ++it;
-                if (rr_in <= rr_stop || it >= maxit) break;
+                if (le_bits(rr_in, rr_stop) || it >= maxit) break;
             }
         }
         if (!alive) break;
@@ -446,7 +493,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
         // u += x; MIXED: an exchange so that the next residual sees the new u
 #pragma unroll
         for (int s = 0; s < NPT; ++s) {
-            const long long n = b0 + threadIdx.x + s * REG_THREADS;
+            const long long n = b0 + tn + s * REG_THREADS;
             if (n < b1) a.u[n] = a.u[n] + (double)x[s];
         }
         if (!MIXED) {
@@ -459,7 +506,7 @@ __global__ void __launch_bounds__(REG_THREADS, 1) k_pcg_reg(RegArgs a) {
     }
 #pragma unroll
     for (int s = 0; s < NPT; ++s) {
-        const long long n = b0 + threadIdx.x + s * REG_THREADS;
+        const long long n = b0 + tn + s * REG_THREADS;
         if (n < b1) a.phi[n] = (bb == 0.0) ? a.g[n] : a.u[n] + a.g[n];
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -768,7 +815,9 @@ static void plan_pcg_reg(Ctx& c) {
     if (G > REG_THREADS) G = REG_THREADS;   // exchange totals: one partial per thread
     if (G > 255) G = 255;          // the fixed-point exchange counts arrivals in 8 bits
     if (G < 1) G = 1;
-    const long long M = (N + G - 1) / G;
+    // (in whole pairs of warps: fewer blocks to exchange among for the same time in each)
+    long long M = (N + G - 1) / G;
+    if (M < REG_THREADS) M = (M + 63) / 64 * 64;
     G = (N + M - 1) / M;           // every block owns at least one node
     const long long npt = (M + REG_THREADS - 1) / REG_THREADS;
     int pick = npt <= 1 ? 1 : npt <= 2 ? 2 : npt <= 4 ? 4 : npt <= 8 ? 8 : 0;
@@ -820,7 +869,10 @@ static void plan_pcg_reg(Ctx& c) {
         const size_t rows_bytes = ((size_t)M * 19 * sizeof(float) + 15) / 16 * 16;
         if (try_plan(true, rows_bytes + (size_t)wpad * sizeof(float))) return;
     }
-    try_plan(false, (size_t)wmax * tsz);
+    const size_t win = (size_t)wmax * tsz, staged = (size_t)std::min<long long>(M, 128) * 19 * tsz;
+    c.pcg_stage = 0;
+    if (!mixed && try_plan(false, win + staged)) c.pcg_stage = (int)std::min<long long>(M, 128);
+    else try_plan(false, win);
 }
 
 static cudaError_t launch_reg(Ctx& c, cudaStream_t st, bool mixed) {
@@ -838,6 +890,8 @@ static cudaError_t launch_reg(Ctx& c, cudaStream_t st, bool mixed) {
                               {-1, 0, 1}, {1, 0, 1}, {0, -1, -1}, {0, 1, -1}, {0, -1, 1}, {0, 1, 1}};
         for (int q = 0; q < 19; ++q) a.woff[q] = d[q][0] + d[q][1] * NX + d[q][2] * NXY;
     }
+    a.stage_rows = c.pcg_stage;
+    a.stage_at = (int)(c.pcg_smem - (size_t)c.pcg_stage * 19 * sizeof(double));
     a.val = c.coop_partial;
     a.arrivals = c.bar64;
     a.fx = c.bar64 + FX_LINE;
