@@ -21,21 +21,6 @@ __global__ void k_bin_caps(int nb, const int* cnt, int* cap, int* cnt_copy);
 __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* total);
 __global__ void k_clamp_counts(Launch L);
 
-struct ObjF {
-    int kind;
-    float a0, a1, a2, a3, a4, a5, a6, a7, a8, a9, a10, a11;
-};
-
-static ObjF obj_f(const Object& o) {
-    ObjF f;
-    f.kind = o.kind;
-    f.a0 = (float)o.a0; f.a1 = (float)o.a1; f.a2 = (float)o.a2;
-    f.a3 = (float)o.a3; f.a4 = (float)o.a4; f.a5 = (float)o.a5;
-    f.a6 = (float)o.a6; f.a7 = (float)o.a7; f.a8 = (float)o.a8;
-    f.a9 = (float)o.a9; f.a10 = (float)o.a10; f.a11 = (float)o.a11;
-    return f;
-}
-
 PF_D float level_set_f(const ObjF& o, float x, float y, float z) {
     if (o.kind == 1) {
         float dx = x - o.a0, dy = y - o.a1, dz = z - o.a2;
@@ -362,25 +347,6 @@ struct PushSmem {
     static_assert(mask % 16 == 0 && stg > mask, "the prefix counts fit in the stages");
     static_assert(sizeof(float4) * TN <= wt, "the node-field tile lands in the deposit tile's room");
 };
-
-// no point of the box [x0, x1) x [y0, y1) x [z0, z1) is in the object, with a margin
-// above the FP32 level set's rounding
-PF_D bool box_clear(const ObjF& o, float x0, float x1, float y0, float y1, float z0, float z1) {
-    if (o.kind == 1) {
-        const float dx = fmaxf(fmaxf(x0 - o.a0, o.a0 - x1), 0.0f), dy = fmaxf(fmaxf(y0 - o.a1, o.a1 - y1), 0.0f),
-                    dz = fmaxf(fmaxf(z0 - o.a2, o.a2 - z1), 0.0f);
-        return dx * dx + dy * dy + dz * dz > o.a3 * 1.0001f + 0.01f;
-    } else if (o.kind == 2) {          // nothing of a cap crater lies above its ground
-        return z0 > o.a0 + 0.01f;
-    } else if (o.kind == 3) {
-        const float l = fminf(o.a0 * x0, o.a0 * x1) + fminf(o.a1 * y0, o.a1 * y1) + fminf(o.a2 * z0, o.a2 * z1);
-        const float big = fmaxf(fabsf(o.a0) * x1 + fabsf(o.a1) * y1 + fabsf(o.a2) * z1, fabsf(o.a3));
-        return l - o.a3 > 1e-4f * big + 0.01f;
-    } else if (o.kind == 4) {          // nor of a raised-rim crater above its rim (its floor is lower)
-        return z0 > fmaxf(o.a6, o.a11) + 0.01f;
-    }
-    return true;
-}
 
 // the whole push of up to 32 particles of the bin that did not simply stay in it (act: the
 // lanes that have one, in slot start + i): as push_one, then the survivors go to the mover

@@ -1,11 +1,46 @@
 """Routes inside the FP64 kernels that must give what the plain route gives.
 
-The PCG sums its dot products in fixed point where the previous totals give a
-scale, and by partial sums where they do not."""
+The push takes a particle's cell, floor and weights from the bits of its
+position and puts the leavers of a bin aside, 256 at a time; the PCG sums its
+dot products in fixed point where the previous totals give a scale, and by
+partial sums where they do not."""
 import numpy as np
 import pytest
 
+from paper_2011_10214_gb300 import workloads as wl
+from tests.pairs import add_species_both, by_id, make_pair
+
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("case", ["sphere16", "ragged"])
+@pytest.mark.parametrize("n,vth", [(1, 0.1), (255, 30.0), (257, 30.0), (1500, 5.0), (4000, 30.0)])
+def test_push_bit_exact_at_cell_edges_and_with_many_leavers(case, n, vth):
+    """One bin at the mesh's corner, full of positions on cell faces, at -0,
+    just below a face and denormal, up to all of them leaving at once."""
+    gpu, orc = make_pair(case, dt=0.3)
+    add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+    g = np.random.default_rng(n)
+    X = g.uniform(0.0, 3.999, (3, n))
+    edge = np.array([-0.0, 0.0, 5e-324, 1e-310, 1.0, 2.0, 3.0, np.nextafter(1.0, 0.0), np.nextafter(4.0, 0.0)])
+    pick = g.integers(0, 4, (3, n)) == 0
+    X[pick] = edge[g.integers(0, len(edge), int(pick.sum()))]
+    V = g.normal(0, vth, (3, n))
+    V[:, ::5] = 0.0
+    ids = np.arange(n, dtype=np.int64)
+    gpu.load_particles(0, X[0], X[1], X[2], V[0], V[1], V[2], ids)
+    orc.load_particles(0, X[0], X[1], X[2], V[0], V[1], V[2], ids)
+    E = wl.random_node_field(orc.mesh.nnodes, 3, scale=0.3)
+    gpu.set_external_E(E); orc.set_external_E(E)
+    for _ in range(3):
+        sg, so = gpu.step(1), orc.step()
+        assert sg["absorbed"][0] == so["absorbed"][0] and sg["pushed"][0] == so["pushed"][0]
+        a, b = by_id(gpu.particles(0)), by_id(orc.P[0])
+        assert np.array_equal(a["id"], b["id"])
+        for k in ("x", "y", "z", "vx", "vy", "vz"):
+            assert np.array_equal(a[k], b[k]), k
+        assert np.array_equal(gpu.node_charge(0), orc.W[0])
+    gpu.close()
 
 
 @pytest.mark.parametrize("n", [(5, 4, 3), (16, 16, 16), (33, 20, 27)])
