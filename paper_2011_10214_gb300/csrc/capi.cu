@@ -412,7 +412,7 @@ void pifepic_destroy(pifepic_ctx* ctx) {
     void* ptrs[] = {c.Lnode, c.ne_row, c.ne_coef, c.ne_qoff, c.ne_q, c.ne_qc, c.ntype, c.gdir, c.lift, c.invdiag, c.invdiagf, c.phi, c.phi_prev, c.u, c.b, c.r, c.p, c.q,
                     c.z ? (void*)(c.z - c.zguard) : nullptr, c.zf ? (void*)(c.zf - c.zguard) : nullptr,
                     c.rf, c.pf, c.qf, c.uf, c.E, c.Ef, c.Wall, c.surfall, c.ctrall, c.imask, c.ibase, c.cell_acc,
-                    c.it_cell, c.it_t, c.it_data, c.it_acc, c.qT, c.cut_cell, c.cut_area, c.qcut, c.patch_node,
+                    c.it_cell, c.it_t, c.it_data, c.it_acc, c.qT, c.cut_cell, c.cut_area, c.patch_node,
                     c.patch_coef, c.patch_coeff, c.red, c.coop_partial, c.rowkind, c.pcg_x, c.ph_tets, c.ph_Q, c.ph_carry, c.ph_cnt, c.ph_base, c.ph_tiles, c.ph_total, c.scal, c.red_ticket, c.bar64, c.err_word, c.inj_dev, c.inj_count,
                     c.inj_base, c.inj_carry, c.next_id};
     for (void* p : ptrs) lib_free(p);
@@ -476,11 +476,11 @@ static pifepic_status encode_tmaps(pifepic_ctx* ctx) {
 static pifepic_status do_setup(pifepic_ctx* ctx) {
     Ctx& c = ctx->c;
     // free a previous interface set-up
-    void* old[] = {c.it_cell, c.it_t, c.it_data, c.it_acc, c.qT, c.cut_cell, c.cut_area, c.qcut,
+    void* old[] = {c.it_cell, c.it_t, c.it_data, c.it_acc, c.qT, c.cut_cell, c.cut_area,
                    c.patch_node, c.patch_coef, c.patch_coeff, c.surfall};
     for (void* p : old) lib_free(p);
     c.it_cell = c.it_t = c.it_acc = c.cut_cell = nullptr;
-    c.it_data = c.qT = c.cut_area = c.qcut = c.patch_coef = nullptr;
+    c.it_data = c.qT = c.cut_area = c.patch_coef = nullptr;
     c.patch_node = nullptr; c.patch_coeff = nullptr; c.surfall = nullptr;
     cudaError_t se = launch_setup(c);
     if (c.bed_outside) FAIL(PIFEPIC_EINVAL, "the bedrock must lie inside the object (a bedrock node has L >= 0)");
@@ -690,8 +690,8 @@ pifepic_status pifepic_add_species(pifepic_ctx* ctx, double qq, double mm, doubl
     q.W = c.Wall + (long long)idx * c.mesh.nnodes;
     q.surf = c.surfall + (long long)idx * (c.ncut > 0 ? c.ncut : 1);
     q.ctr = c.ctrall + idx * NCTR;
-    ALLOC(q.mov_n, 2 * sizeof(unsigned long long));
-    CUDA_OK(szero(c.stream, q.mov_n, 2 * sizeof(unsigned long long)));
+    ALLOC(q.mov_n, 3 * sizeof(unsigned long long));
+    CUDA_OK(szero(c.stream, q.mov_n, 3 * sizeof(unsigned long long)));
     pifepic_status st = ensure_movers(ctx, idx, 1 << 16);
     if (st) return st;
     // empty bins

@@ -32,20 +32,19 @@ __constant__ TetTables cTf;
 __constant__ float cFold[2][81];
 
 // ---- right-hand side ----------------------------------------------------------
-__global__ void k_qcut(RhsArgs a, const double* area, double* qcut) {
-    long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (c >= a.ncut) return;
-    double Q = 0.0;
-    int ns = *a.nspec;
-    for (int s = 0; s < ns; ++s) Q = Q + a.coefs[s] * (double)(long long)a.surf[(long long)s * a.ncut + c];
-    qcut[c] = -(Q / area[c]);
-}
-
-__global__ void k_qtets(long long nit, const int* it_acc, const double* qcut, double* qT) {
+// the surface charge density of each interface tet's object, from its cut cell
+__global__ void k_qtets(long long nit, const int* it_acc, RhsArgs a, const double* area, double* qT) {
     long long T = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (T >= nit) return;
-    int a = it_acc[T];
-    qT[T] = a >= 0 ? qcut[a] : 0.0;
+    const int c = it_acc[T];
+    double q = 0.0;
+    if (c >= 0) {
+        double Q = 0.0;
+        int ns = *a.nspec;
+        for (int s = 0; s < ns; ++s) Q = Q + a.coefs[s] * (double)(long long)a.surf[(long long)s * a.ncut + c];
+        q = -(Q / area[c]);
+    }
+    qT[T] = q;
 }
 
 // the flux-jump terms of a node's right-hand side (the node rows of the set-up)
@@ -56,15 +55,42 @@ struct FluxRows {
     const double* qc;
 };
 
+// The solve's start vector: the last potential, or once two earlier solves exist
+// its linear extrapolation 2 phi_{n-1} - phi_{n-2} (particles move the charge
+// smoothly from step to step, so this start is closer), less the Dirichlet
+// values; phi_prev <- phi.  The solve still stops on the same relative residual.
+struct StartArgs {
+    const double* phi;
+    double* phi_prev;
+    const double* g;
+    double* u;                // null: the start goes into the box of the fast-diagonalisation solve
+    const long long* hist;    // solves before this one (3: three or more; counted by the node field's kernel)
+    FdPlan d;
+};
+static __device__ __forceinline__ void start_vector(const StartArgs& a, const Mesh& m, long long n, bool dirichlet) {
+    const double p = a.phi[n];
+    const double start = *a.hist >= 2 ? 2.0 * p - a.phi_prev[n] : p;
+    if (a.u) {
+        a.u[n] = dirichlet ? 0.0 : start - a.g[n];
+    } else {
+        int i, j, k;
+        node_ijk(m, n, i, j, k);
+        i -= a.d.x0; j -= a.d.y0; k -= a.d.z0;
+        if ((unsigned)i < (unsigned)a.d.mx && (unsigned)j < (unsigned)a.d.my && (unsigned)k < (unsigned)a.d.mz)
+            a.d.u[k * a.d.PV + j * a.d.ldv + i] = start - a.g[n];
+    }
+    a.phi_prev[n] = p;
+}
+
+// right-hand side, and the start vector in the same pass (START)
+template <bool START>
 __global__ void k_rhs(FieldArgs f, RhsArgs a, FluxRows fr, const double* qT, const double* lift, double* b,
-                      const double* Fext, long long* hist) {
+                      const double* Fext, const __grid_constant__ StartArgs start) {
     const Mesh& m = f.m;
     long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    // solves so far, this one included (capped at 3): the start-vector kernel
-    // that follows extrapolates only once two earlier solves exist
-    if (hist && n == 0 && *hist < 3) *hist += 1;
     if (n >= m.nnodes) return;
     int ty = f.ntype[n];
+    if (START) start_vector(start, m, n, ty == -3);
     if (ty == -3) { b[n] = 0.0; return; }
     double F = 0.0;
     if (Fext) {
@@ -84,6 +110,11 @@ __global__ void k_rhs(FieldArgs f, RhsArgs a, FluxRows fr, const double* qT, con
     b[n] = F - lift[n];
 }
 
+// one more solve done (k_node_E and k_node_E_f: the last kernel of every solve)
+static __device__ __forceinline__ void count_solve(long long* hist) {
+    if (hist && *hist < 3) *hist += 1;
+}
+
 // ---- PCG kernels ------------------------------------------------------------------
 __global__ void k_matvec(FieldArgs f, const double* x, double* y) {
     long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -98,20 +129,6 @@ __global__ void k_phi_from_u(long long N, const double* u, const double* g, doub
     long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (n < N) phi[n] = S->bb == 0.0 ? g[n] : u[n] + g[n];
 }
-// PCG start vector: the last potential, or once two earlier solves exist its
-// linear extrapolation 2 phi_{n-1} - phi_{n-2} (particles move the charge
-// smoothly from step to step, so this start is closer); phi_prev <- phi.  The
-// solve still stops on the same relative residual.
-__global__ void k_u_from_phi(long long N, const int* ntype, const double* phi, double* phi_prev, const double* g,
-                             double* u, const long long* hist) {
-    long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const double p = phi[n];
-    const double start = (*hist >= 3) ? 2.0 * p - phi_prev[n] : p;
-    u[n] = ntype[n] == -3 ? 0.0 : start - g[n];
-    phi_prev[n] = p;
-}
-
 // ---- node field ---------------------------------------------------------------------
 // Minus the volume-weighted mean of the element gradients around a node, the
 // plasma-side pieces if there are any.  A block takes 4 x 4 x 4 nodes: first each
@@ -124,7 +141,7 @@ __global__ void k_u_from_phi(long long N, const int* ntype, const double* phi, d
 constexpr int N64_T = 4, N64_C = N64_T + 1, N64_TETS = N64_C * N64_C * N64_C * 5, N64_GRAD = 13;
 __global__ void __launch_bounds__(256) k_node_E(FieldArgs f, const double* L, const unsigned char* imask, const int* ibase,
                                                 const double* it_data, const double* qT, const double* phi, double4* E,
-                                                float4* Ef) {
+                                                float4* Ef, long long* hist) {
     enum { APL = 0, VPL = 3, AAL = 4, VAL = 7 };
     __shared__ double ct[8][N64_TETS];
     __shared__ double res[8][N64_T * N64_T * N64_T];
@@ -133,6 +150,7 @@ __global__ void __launch_bounds__(256) k_node_E(FieldArgs f, const double* L, co
     const Mesh& m = f.m;
     const int tid = threadIdx.x;
     const int i0 = blockIdx.x * N64_T, j0 = blockIdx.y * N64_T, k0 = blockIdx.z * N64_T;
+    if (tid == 0 && i0 + j0 + k0 == 0) count_solve(hist);
     if (tid < 120) grad[(tid / 12) * N64_GRAD + tid % 12] = (&cTf.grad[0][0][0][0])[tid];
     else if (tid >= 128 && tid < 133) vol[tid - 128] = cTf.vol[tid - 128];
     else if (tid >= 160 && tid < 200) vert[tid - 160] = (&cTf.vert[0][0][0])[tid - 160];
@@ -228,10 +246,10 @@ __global__ void __launch_bounds__(256) k_node_E(FieldArgs f, const double* L, co
     if (Ef) Ef[n] = make_float4((float)e.x, (float)e.y, (float)e.z, 0.0f);
 }
 
-static void launch_node_E(const FieldArgs& f, const Ctx& c, float4* Ef, cudaStream_t st) {
+static void launch_node_E(const FieldArgs& f, const Ctx& c, float4* Ef, long long* hist, cudaStream_t st) {
     const Mesh& m = c.mesh;
     const dim3 grid((m.NX + N64_T - 1) / N64_T, (m.NY + N64_T - 1) / N64_T, (m.NZ + N64_T - 1) / N64_T);
-    k_node_E<<<grid, 256, 0, st>>>(f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi, c.E, Ef);
+    k_node_E<<<grid, 256, 0, st>>>(f, c.Lnode, c.imask, c.ibase, c.it_data, c.qT, c.phi, c.E, Ef, hist);
 }
 
 // Node field in FP32 (MIXED steps; the push reads only this copy).  Same
@@ -247,12 +265,13 @@ constexpr int NE_FOLD = 97;   // the parity tables' stride in shared memory (not
 __global__ void __launch_bounds__(NE_BX * NE_BY * NE_BZ) k_node_E_f(Mesh m, const int* row, long long R,
                                                                     const float* coef, const int* qoff,
                                                                     const int4* qent, const double* qT,
-                                                                    const double* phi, float4* Ef) {
+                                                                    const double* phi, float4* Ef, long long* hist) {
     __shared__ float ph[NE_TX * NE_TY * NE_TZ];
     __shared__ float sF[2 * NE_FOLD];
     const int i0 = blockIdx.x * NE_BX, j0 = blockIdx.y * NE_BY, k0 = blockIdx.z * NE_BZ;
     const int tid = threadIdx.x + NE_BX * (threadIdx.y + NE_BY * threadIdx.z);
     const int i = i0 + threadIdx.x, j = j0 + threadIdx.y, k = k0 + threadIdx.z;
+    if (tid == 0 && i0 + j0 + k0 == 0) count_solve(hist);
     const bool mine = i < m.NX && j < m.NY && k < m.NZ;
     const long long n = mine ? node_id(m, i, j, k) : 0;
     const int r = mine ? row[n] : -1;
@@ -299,11 +318,11 @@ __global__ void __launch_bounds__(NE_BX * NE_BY * NE_BZ) k_node_E_f(Mesh m, cons
     Ef[n] = make_float4(e0, e1, e2, 0.f);
 }
 
-static void launch_node_E_f(const Ctx& c, cudaStream_t st) {
+static void launch_node_E_f(const Ctx& c, long long* hist, cudaStream_t st) {
     const Mesh& m = c.mesh;
     dim3 grid((m.NX + NE_BX - 1) / NE_BX, (m.NY + NE_BY - 1) / NE_BY, (m.NZ + NE_BZ - 1) / NE_BZ);
     k_node_E_f<<<grid, dim3(NE_BX, NE_BY, NE_BZ), 0, st>>>(m, c.ne_row, c.ne_nrows, c.ne_coef, c.ne_qoff, c.ne_q,
-                                                          c.qT, c.phi, c.Ef);
+                                                          c.qT, c.phi, c.Ef, hist);
 }
 
 
@@ -372,33 +391,26 @@ cudaError_t launch_E_to_pic(const Ctx& c, cudaStream_t st, bool both) {
     return cudaGetLastError();
 }
 
-// the solve's start vector, where its solver keeps it
-cudaError_t launch_fd_start(Ctx& c, cudaStream_t st);        // pcg_fd.cu
-cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
-static cudaError_t launch_start(Ctx& c, cudaStream_t st, bool fd) {
-    if (fd) return launch_fd_start(c, st);
-    k_u_from_phi<<<nb(c.mesh.nnodes), 256, 0, st>>>(c.mesh.nnodes, c.ntype, c.phi, c.phi_prev, c.gdir, c.u,
-                                                    solve_hist(c));
+cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);   // pcg_fd.cu
+// q_T, right-hand side and start vector (where the solver keeps it)
+static cudaError_t launch_rhs(Ctx& c, cudaStream_t st, bool fd, const double* Fext) {
+    const long long N = c.mesh.nnodes;
+    const RhsArgs a = rargs(c);
+    if (!Fext && c.nit > 0) k_qtets<<<nb(c.nit), 256, 0, st>>>(c.nit, c.it_acc, a, c.cut_area, c.qT);
+    const StartArgs start{c.phi, c.phi_prev, c.gdir, fd ? nullptr : c.u, solve_hist(c), c.fd};
+    k_rhs<true><<<node_blocks(N), node_threads(N), 0, st>>>(fargs(c), a, flux_rows(c), c.qT, c.lift, c.b, Fext, start);
     return cudaGetLastError();
 }
 
 static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     FieldArgs f = fargs(c);
-    RhsArgs a = rargs(c);
-    long long N = c.mesh.nnodes;
-    if (!Fext) {
-        if (c.ncut > 0) k_qcut<<<nb(c.ncut), 256, 0, st>>>(a, c.cut_area, c.qcut);
-        if (c.nit > 0) k_qtets<<<nb(c.nit), 256, 0, st>>>(c.nit, c.it_acc, c.qcut, c.qT);
-    }
-    k_rhs<<<node_blocks(N), node_threads(N), 0, st>>>(f, a, flux_rows(c), c.qT, c.lift, c.b, Fext,
-                                                       solve_hist(c));
     const bool fd = Fext ? c.fd_ready : c.fd_single;
-    cudaError_t e = launch_start(c, st, fd);
+    cudaError_t e = launch_rhs(c, st, fd, Fext);
     if (e != cudaSuccess) return e;
     e = fd ? launch_pcg_fd(c, st) : launch_pcg_coop(c, st);
     if (e != cudaSuccess) return e;
-    if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, st);
-    else launch_node_E(f, c, c.Ef, st);
+    if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, solve_hist(c), st);
+    else launch_node_E(f, c, c.Ef, solve_hist(c), st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_E_to_pic(c, st, c.precision != PIFEPIC_MIXED);
@@ -406,27 +418,18 @@ static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
 
 // the solve's pieces around the PCG, for the batched step (batch.cu); fd: the
 // member's solve is the fast-diagonalisation one
-cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st, bool fd) {
-    FieldArgs f = fargs(c);
-    RhsArgs a = rargs(c);
-    long long N = c.mesh.nnodes;
-    if (c.ncut > 0) k_qcut<<<nb(c.ncut), 256, 0, st>>>(a, c.cut_area, c.qcut);
-    if (c.nit > 0) k_qtets<<<nb(c.nit), 256, 0, st>>>(c.nit, c.it_acc, c.qcut, c.qT);
-    k_rhs<<<node_blocks(N), node_threads(N), 0, st>>>(f, a, flux_rows(c), c.qT, c.lift, c.b, nullptr,
-                                                       solve_hist(c));
-    return launch_start(c, st, fd);
-}
+cudaError_t launch_solve_prefix(Ctx& c, cudaStream_t st, bool fd) { return launch_rhs(c, st, fd, nullptr); }
 cudaError_t launch_solve_suffix(Ctx& c, cudaStream_t st) {
     FieldArgs f = fargs(c);
-    if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, st);
-    else launch_node_E(f, c, c.Ef, st);
+    if (c.precision == PIFEPIC_MIXED) launch_node_E_f(c, solve_hist(c), st);
+    else launch_node_E(f, c, c.Ef, solve_hist(c), st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_E_to_pic(c, st, c.precision != PIFEPIC_MIXED);
 }
 
 // kernels launched per solve
-int solve_graph_fixed_kernels(const Ctx& c) { return (c.ncut > 0) + (c.nit > 0) + 4 + (c.refine > 1); }
+int solve_graph_fixed_kernels(const Ctx& c) { return (c.nit > 0) + 3 + (c.refine > 1); }
 
 // The solve as one CUDA graph (both precisions): q_T -> RHS -> warm start ->
 // persistent PCG -> node field
@@ -638,7 +641,7 @@ cudaError_t queue_stats(Ctx* const* c, int n, cudaStream_t st) {
 // FP64 node field from the current phi into E only (the FP32 copy the MIXED
 // push reads is left as the step made it)
 cudaError_t launch_node_E64(Ctx& c) {
-    launch_node_E(fargs(c), c, nullptr, c.stream);
+    launch_node_E(fargs(c), c, nullptr, nullptr, c.stream);
     return cudaGetLastError();
 }
 
@@ -675,13 +678,6 @@ cudaError_t set_field_tables(const TetTables& t) {
     cudaError_t e = cudaMemcpyToSymbol(cTf, &t, sizeof(TetTables));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(cFold, Ff, sizeof(Ff));
     return e;
-}
-
-cudaError_t launch_qtets(Ctx& c) {
-    RhsArgs a = rargs(c);
-    if (c.ncut > 0) k_qcut<<<nb(c.ncut), 256, 0, c.stream>>>(a, c.cut_area, c.qcut);
-    if (c.nit > 0) k_qtets<<<nb(c.nit), 256, 0, c.stream>>>(c.nit, c.it_acc, c.qcut, c.qT);
-    return cudaGetLastError();
 }
 
 // ======================================================================================
@@ -844,7 +840,7 @@ pifepic_status solve_field_noalloc(Ctx& c, const double* F, const double* q, dou
     unsigned gb = nb(N);
     cudaStream_t st = c.stream;
     k_na_state<<<1, 1, 0, st>>>(S, ticket, c.tol * c.tol, c.maxit);
-    k_rhs<<<gb, 256, 0, st>>>(f, a, flux_rows(c), q, c.lift, bvec, F, nullptr);
+    k_rhs<false><<<gb, 256, 0, st>>>(f, a, flux_rows(c), q, c.lift, bvec, F, StartArgs{});
     cudaMemsetAsync(u, 0, sizeof(double) * N, st);
     k_matvec<<<gb, 256, 0, st>>>(f, u, qv);
     k_na_init<<<gb, 256, 0, st>>>(f, bvec, qv, r, p, partial, ticket, S);

@@ -100,6 +100,7 @@ struct SpeciesDev {
     PArrF movF_in, movF_out;
     unsigned long long* mov_in_n;   // counters (device)
     unsigned long long* mov_out_n;
+    unsigned long long* mov_read;   // blocks that have read the waiting list this step
     long long mcap;
     unsigned long long* W;          // [nnodes] fixed-point charge
     unsigned long long* surf;       // [ncut] collected macro-particles
@@ -155,7 +156,7 @@ struct Species {
     int* bcap = nullptr;
     int* bcount = nullptr;
     int* bstay = nullptr;
-    unsigned long long* mov_n = nullptr;   // [2]
+    unsigned long long* mov_n = nullptr;   // [3]: waiting, this step's movers, arrivals of the list's readers
     unsigned long long* W = nullptr;
     unsigned long long* surf = nullptr;
     unsigned long long* ctr = nullptr;
@@ -283,7 +284,6 @@ struct Ctx {
     long long ncut = 0;
     int* cut_cell = nullptr;
     double* cut_area = nullptr;
-    double* qcut = nullptr;
     // patch rows
     long long npatch = 0;
     long long* patch_node = nullptr;

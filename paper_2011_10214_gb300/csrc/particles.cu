@@ -357,6 +357,15 @@ __global__ void __launch_bounds__(256) k_push_bins(const __grid_constant__ Launc
     if (tid < NCTR && sctr[tid]) atomicAdd(&S.ctr[tid], (unsigned long long)sctr[tid]);
 }
 
+// before a step's push: no charge on the nodes, no movers yet (one launch for both)
+__global__ void k_push_prep(Launch L, unsigned long long* W, long long words) {
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t0 < L.nspecies) *L.sp[t0].mov_out_n = 0ull;
+    for (long long q = t0; q < words / 2; q += (long long)gridDim.x * blockDim.x)
+        reinterpret_cast<ulonglong2*>(W)[q] = make_ulonglong2(0ull, 0ull);
+    if (t0 == 0 && (words & 1)) W[words - 1] = 0ull;
+}
+
 // particles waiting in the mover list (spilled last step): same arithmetic,
 // node field read from global memory; every survivor goes back to the list
 // of this step's movers
@@ -403,24 +412,40 @@ __global__ void k_push_movers(Launch L) {
     }
     __syncthreads();
     if (threadIdx.x < NCTR && sctr[threadIdx.x]) atomicAdd(&S.ctr[threadIdx.x], sctr[threadIdx.x]);
+    list_read(S);
 }
 
 // ------------------------------------------------------------------------------------
 // injection (reading of Sec. 3.1.3 / Sec. 5.2.2; see inject_one)
 // ------------------------------------------------------------------------------------
 // count = floor(carry + rate) per stream, ids consecutive per species in face order
+// (one warp, a stream per lane: serial over the streams it took 8 us of FP64 and memory latency)
 __global__ void k_inject_counts(InjArgs a) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int q = 0; q < a.nst; ++q) {
-        const InjectDev& d = a.st[q];
-        double cr = a.carry[q] + d.rate;
-        double nf = floor(cr);
-        a.carry[q] = cr - nf;
-        int cnt = (int)nf;
-        if (cnt > d.maxcnt) cnt = d.maxcnt;
-        a.count[q] = cnt;
-        a.idbase[q] = a.next_id[d.species];
-        a.next_id[d.species] += cnt;
+    const int lane = threadIdx.x;
+    for (int q0 = 0; q0 < a.nst; q0 += 32) {
+        const int q = q0 + lane;
+        int cnt = 0, sp = -1;
+        long long base = 0;
+        if (q < a.nst) {
+            const InjectDev& d = a.st[q];
+            sp = d.species;
+            base = a.next_id[sp];
+            double cr = a.carry[q] + d.rate;
+            double nf = floor(cr);
+            a.carry[q] = cr - nf;
+            cnt = (int)nf;
+            if (cnt > d.maxcnt) cnt = d.maxcnt;
+            a.count[q] = cnt;
+        }
+        bool last = sp >= 0;
+        for (int o = 0; o < 32; ++o) {
+            const int so = __shfl_sync(0xffffffffu, sp, o), co = __shfl_sync(0xffffffffu, cnt, o);
+            if (so == sp && o < lane) base += co;
+            if (so == sp && o > lane) last = false;
+        }
+        if (q < a.nst) a.idbase[q] = base;
+        if (last) a.next_id[sp] = base + cnt;
+        __syncwarp();
     }
 }
 
@@ -501,13 +526,13 @@ __global__ void k_rebin(Launch L) {
     }
 }
 
-__global__ void k_step_advance(long long* step) { *step += 1; }
-
-__global__ void k_clamp_counts(Launch L) {
+// (step: the counter of steps, advanced at the end of one; or null)
+__global__ void k_clamp_counts(Launch L, long long* step) {
     const int s = blockIdx.y;
     const SpeciesDev& S = L.sp[s];
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < L.nblocks && S.bcount[b] > S.bcap[b]) S.bcount[b] = S.bcap[b];
+    if (b == 0 && s == 0 && step) *step += 1;
     if (b == 0) {
         unsigned long long sp = *S.mov_in_n;
         S.ctr[C_SPILLED] = sp < (unsigned long long)S.mcap ? sp : (unsigned long long)S.mcap;
@@ -713,7 +738,7 @@ Launch make_launch(Ctx& c) {
         d.bstart = q.bstart; d.bcap = q.bcap; d.bcount = q.bcount; d.bstay = q.bstay;
         d.mov_in = q.mov[0]; d.mov_out = q.mov[1];
         d.movF_in = q.movF[0]; d.movF_out = q.movF[1];
-        d.mov_in_n = q.mov_n; d.mov_out_n = q.mov_n + 1;
+        d.mov_in_n = q.mov_n; d.mov_out_n = q.mov_n + 1; d.mov_read = q.mov_n + 2;
         d.mcap = q.mcap;
         d.W = q.W; d.surf = q.surf; d.ctr = q.ctr;
         d.reflect = q.reflect;
@@ -785,7 +810,7 @@ cudaError_t launch_build_bins(Ctx& c, int s, PArr flat, long long n, bool) {
     L = make_launch(c);
     cudaMemsetAsync(q.mov_n, 0, 2 * sizeof(unsigned long long), c.stream);
     if (n > 0) k_bin_scatter<<<nb(n), 256, 0, c.stream>>>(L, s, flat, n, c.track != 0);
-    k_clamp_counts<<<dim3(nb(c.nblocks), (unsigned)c.sp.size()), 256, 0, c.stream>>>(L);
+    k_clamp_counts<<<dim3(nb(c.nblocks), (unsigned)c.sp.size()), 256, 0, c.stream>>>(L, nullptr);
     e = cudaStreamSynchronize(c.stream);
     lib_free(cnt);
     lib_free(tot);
@@ -817,10 +842,11 @@ cudaError_t launch_half_kick(Ctx& c) {
 // push of all bins (+ node-field tiles by TMA) and of waiting movers
 // what precedes a push: the step's mover-list counts and node charges start at zero
 cudaError_t launch_push_prep(Ctx& c) {
-    int ns = (int)c.sp.size();
-    for (int s = 0; s < ns; ++s)
-        cudaMemsetAsync(c.sp[s].mov_n + 1, 0, sizeof(unsigned long long), c.stream);
-    cudaMemsetAsync(c.Wall, 0, sizeof(unsigned long long) * ns * c.mesh.nnodes, c.stream);
+    Launch L = make_launch(c);
+    const long long words = (long long)L.nspecies * c.mesh.nnodes;
+    const long long blocks = (words / 2 + 255) / 256;
+    k_push_prep<<<(unsigned)(blocks < 1 ? 1 : blocks > 8 * 152 ? 8 * 152 : blocks), 256, 0, c.stream>>>(L, c.Wall, words);
+    c.launches += 1;
     return cudaGetLastError();
 }
 
@@ -952,11 +978,9 @@ cudaError_t launch_inject(Ctx& c) {
 cudaError_t launch_rebin(Ctx& c) {
     Launch L = make_launch(c);
     int ns = (int)c.sp.size();
-    for (int s = 0; s < ns; ++s) cudaMemsetAsync(c.sp[s].mov_n, 0, sizeof(unsigned long long), c.stream);
     k_rebin<<<dim3(4 * 152, ns), 256, 0, c.stream>>>(L);
-    k_clamp_counts<<<dim3(nb(c.nblocks), ns), 256, 0, c.stream>>>(L);
-    k_step_advance<<<1, 1, 0, c.stream>>>((long long*)(c.scal + 42));
-    c.launches += 3;
+    k_clamp_counts<<<dim3(nb(c.nblocks), ns), 256, 0, c.stream>>>(L, (long long*)(c.scal + 42));
+    c.launches += 2;
     return cudaGetLastError();
 }
 

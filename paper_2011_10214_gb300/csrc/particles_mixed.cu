@@ -19,7 +19,8 @@ namespace pf {
 __global__ void k_bin_count(Launch L, PArr a, long long n, int* cnt);
 __global__ void k_bin_caps(int nb, const int* cnt, int* cap, int* cnt_copy);
 __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* total);
-__global__ void k_clamp_counts(Launch L);
+__global__ void k_clamp_counts(Launch L, long long* step);
+cudaError_t launch_push_prep(Ctx& c);
 
 PF_D float level_set_f(const ObjF& o, float x, float y, float z) {
     if (o.kind == 1) {
@@ -689,6 +690,7 @@ __global__ void k_push_movers_m(Launch L, ObjF of, float dthf) {
     }
     __syncthreads();
     if (threadIdx.x < NCTR && sctr[threadIdx.x]) atomicAdd(&S.ctr[threadIdx.x], sctr[threadIdx.x]);
+    list_read(S);
 }
 
 // injection: FP32 sampling (same random streams as the FP64 path) and FP32
@@ -954,7 +956,6 @@ static InjArgs inj_args_m(Ctx& c) {
 }
 
 __global__ void k_inject_counts(InjArgs a);   // particles.cu
-__global__ void k_step_advance(long long* step);
 
 // one push launch; the kernel's dynamic shared-memory limit is raised once to what it
 // needs (above the 48 KB default)
@@ -985,12 +986,7 @@ static cudaError_t push_bins_by_fill(dim3 grid, cudaStream_t st, const Launch& L
 }
 
 // what precedes a push: the step's mover-list counts and node charges start at zero
-cudaError_t launch_push_prep_mixed(Ctx& c) {
-    int ns = (int)c.sp.size();
-    for (int s = 0; s < ns; ++s) cudaMemsetAsync(c.sp[s].mov_n + 1, 0, sizeof(unsigned long long), c.stream);
-    cudaMemsetAsync(c.Wall, 0, sizeof(unsigned long long) * ns * c.mesh.nnodes, c.stream);
-    return cudaGetLastError();
-}
+cudaError_t launch_push_prep_mixed(Ctx& c) { return launch_push_prep(c); }
 
 cudaError_t launch_push_mixed(Ctx& c) {
     cudaError_t e = launch_push_prep_mixed(c);
@@ -1152,17 +1148,15 @@ __global__ void k_deposit_arrivals_m(Launch L) {
 cudaError_t launch_rebin_mixed(Ctx& c) {
     Launch L = make_launch(c);
     int ns = (int)c.sp.size();
-    for (int s = 0; s < ns; ++s) cudaMemsetAsync(c.sp[s].mov_n, 0, sizeof(unsigned long long), c.stream);
     const bool defer = c.refine == 1;   // (a finer IFE mesh takes the deposits node by node)
     if (defer) k_rebin_m<true><<<dim3(4 * 152, ns), 256, 0, c.stream>>>(L);
     else k_rebin_m<false><<<dim3(4 * 152, ns), 256, 0, c.stream>>>(L);
-    k_clamp_counts<<<dim3(nb(c.nblocks), ns), 256, 0, c.stream>>>(L);
+    k_clamp_counts<<<dim3(nb(c.nblocks), ns), 256, 0, c.stream>>>(L, (long long*)(c.scal + 42));
     if (defer) {
         if (c.bin_edge == 8) k_deposit_arrivals_m<8><<<dim3(c.nblocks, ns), 256, 0, c.stream>>>(L);
         else k_deposit_arrivals_m<4><<<dim3(c.nblocks, ns), 256, 0, c.stream>>>(L);
     }
-    k_step_advance<<<1, 1, 0, c.stream>>>((long long*)(c.scal + 42));
-    c.launches += defer ? 4 : 3;
+    c.launches += defer ? 3 : 2;
     return cudaGetLastError();
 }
 
@@ -1253,7 +1247,7 @@ cudaError_t launch_build_bins_mixed(Ctx& c, int s, PArr flat, long long n, bool)
     L = make_launch(c);
     cudaMemsetAsync(q.mov_n, 0, 2 * sizeof(unsigned long long), c.stream);
     if (n > 0) k_bin_scatter_m<<<nb(n), 256, 0, c.stream>>>(L, s, flat, n, c.track != 0);
-    k_clamp_counts<<<dim3(nb(c.nblocks), (unsigned)c.sp.size()), 256, 0, c.stream>>>(L);
+    k_clamp_counts<<<dim3(nb(c.nblocks), (unsigned)c.sp.size()), 256, 0, c.stream>>>(L, nullptr);
     e = cudaStreamSynchronize(c.stream);
     lib_free(cnt);
     lib_free(tot);

@@ -745,26 +745,6 @@ __global__ void k_fd_box(Mesh m, const double* invdiag, const int* ntype, FdPlan
     s[e] = sv;
 }
 
-// the start vector in the box (as k_u_from_phi): the last potential, or once two
-// earlier solves exist its linear extrapolation, less the Dirichlet values; phi_prev <- phi
-__global__ void k_fd_start(Mesh m, FdPlan d, const double* phi, double* phi_prev, const double* g,
-                           const long long* hist) {
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= m.nnodes) return;
-    const double p = phi[n];
-    int i, j, k;
-    node_ijk(m, n, i, j, k);
-    i -= d.x0; j -= d.y0; k -= d.z0;
-    if ((unsigned)i < (unsigned)d.mx && (unsigned)j < (unsigned)d.my && (unsigned)k < (unsigned)d.mz)
-        d.u[k * d.PV + j * d.ldv + i] = ((*hist >= 3) ? 2.0 * p - phi_prev[n] : p) - g[n];
-    phi_prev[n] = p;
-}
-cudaError_t launch_fd_start(Ctx& c, cudaStream_t st) {
-    k_fd_start<<<(unsigned)((c.mesh.nnodes + 255) / 256), 256, 0, st>>>(c.mesh, c.fd, c.phi, c.phi_prev, c.gdir,
-                                                                        (const long long*)(c.scal + 43));
-    return cudaGetLastError();
-}
-
 // eigenvector k (node index j counted from the face) of K v = lambda M v on n
 // cells: sines from a Dirichlet end, cosines from a Neumann end, half-integer
 // wave numbers where the ends differ; M-orthonormal

@@ -9,6 +9,16 @@ namespace pf {
 
 constexpr int MAX_TRIES = 32;
 
+// end of a kernel over the species' waiting list (a block per blockIdx.x): the
+// last block to have read it empties it, for the rebin's spills
+PF_D void list_read(const SpeciesDev& S) {
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(S.mov_read, 1ull) == gridDim.x - 1) {
+        *S.mov_in_n = 0ull;
+        *S.mov_read = 0ull;
+    }
+}
+
 struct InjArgs {
     const InjectDev* st;
     int nst;

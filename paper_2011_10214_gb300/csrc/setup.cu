@@ -656,8 +656,6 @@ cudaError_t launch_setup(Ctx& c) {
         nc = c.ncut > 0 ? c.ncut : 1;
         CK(lib_malloc(&c.cut_cell, sizeof(int) * nc));
         CK(lib_malloc(&c.cut_area, sizeof(double) * nc));
-        CK(lib_malloc(&c.qcut, sizeof(double) * nc));
-        CK(cudaMemsetAsync(c.qcut, 0, sizeof(double) * nc, st));
     }
     k_cut_list<<<nb(m.ncells), 256, 0, st>>>(m, flag, scan, carea, c.cut_cell, c.cut_area, own);
     k_cell_acc<<<nb(m.ncells), 256, 0, st>>>(m, own, c.cell_acc);
