@@ -3,6 +3,8 @@
 // the 5-tet P1 stencil, explicit 19-slot rows where a node touches an interface
 // tet) and deterministic block / grid reductions.
 #pragma once
+#include <type_traits>
+
 #include "internal.h"
 
 namespace pf {
@@ -292,25 +294,40 @@ static __device__ __forceinline__ void node_ijk(const Mesh& m, long long n, int&
     k = (int)kk;
 }
 
-// ---- deterministic block reduction of NV doubles -----------------------------
+// ---- deterministic block reductions -------------------------------------------
+// The FP64 block sum of NV <= 4 values (thread 0 gets the totals).  An FP64 add
+// takes a scheduler 67 cycles, so the values share the butterfly: a lane keeps
+// half of them at each of the first steps, 5 adds a warp for one or two values
+// and 6 for three or four, and one warp takes the warps' sums together.  (Five
+// adds a value in every warp: an exchange of three values took 5 us, now 3.)
+// sh: 4 doubles a warp.
 template <int NV>
-static __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
-    // sh: [NV][32]
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double s = v[q];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) sh[q * 32 + w] = s;
+static __device__ __forceinline__ void block_sum_f64(double (&v)[NV], double* sh) {
+    static_assert(NV <= 4, "four values at most");
+    constexpr int P = NV == 1 ? 1 : NV == 2 ? 2 : 4;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double s = v[0];
+    if (P == 2) {
+        const bool up = lane & 16;
+        s = (up ? v[NV - 1] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[NV - 1], 16);
+    } else if (P == 4) {
+        const double v3 = NV == 4 ? v[NV - 1] : 0.0, v1 = v[NV > 1 ? 1 : 0], v2 = v[NV > 2 ? 2 : 0];
+        const bool up = lane & 16, odd = lane & 8;
+        const double s0 = (up ? v2 : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v2, 16);
+        const double s1 = (up ? v3 : v1) + __shfl_xor_sync(0xffffffffu, up ? v1 : v3, 16);
+        s = (odd ? s1 : s0) + __shfl_xor_sync(0xffffffffu, odd ? s0 : s1, 8);
     }
+#pragma unroll
+    for (int o = 16 / P; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane % (32 / P) == 0) sh[w * P + lane / (32 / P)] = s;
     __syncthreads();
     if (w == 0) {
+        s = 0.0;
+        for (int k = lane; k < nw * P; k += 32) s += sh[k];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = lane < nw ? sh[q * 32 + lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-            v[q] = s;
-        }
+        for (int o = P; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) v[q] = __shfl_sync(0xffffffffu, s, q);
     }
     __syncthreads();
 }
@@ -320,6 +337,10 @@ static __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
 // instruction only every few dozen cycles on this part
 template <typename A, int NV>
 static __device__ __forceinline__ void block_sum_t(A (&v)[NV], A* sh) {
+    if constexpr (std::is_same<A, double>::value && NV <= 4) {
+        block_sum_f64<NV>(v, sh);
+        return;
+    }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -369,7 +390,7 @@ template <int NV>
 static __device__ __forceinline__ bool grid_sum(double (&v)[NV], double* partial, unsigned* ticket, double (&tot)[NV]) {
     __shared__ double sh[NV * 32];
     __shared__ bool last;
-    block_sum<NV>(v, sh);
+    block_sum_f64<NV>(v, sh);
     if (threadIdx.x == 0) {
         for (int q = 0; q < NV; ++q) partial[(long long)q * gridDim.x + blockIdx.x] = v[q];
         __threadfence();
@@ -385,7 +406,7 @@ static __device__ __forceinline__ bool grid_sum(double (&v)[NV], double* partial
         for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
             s[q] += ((volatile double*)partial)[(long long)q * gridDim.x + b];
     }
-    block_sum<NV>(s, sh);
+    block_sum_f64<NV>(s, sh);
     if (threadIdx.x == 0) {
         for (int q = 0; q < NV; ++q) tot[q] = s[q];
         *ticket = 0;

@@ -718,7 +718,7 @@ __global__ void k_fd_profile(Mesh m, const double* invdiag, FdPlan d, double* pr
     double v[1] = {0.0};
     for (int e = threadIdx.x; e < d.mx * d.my; e += blockDim.x)
         v[0] += fd_eps(m, invdiag, d.x0 + e % d.mx, d.y0 + e / d.mx, d.z0 + (int)blockIdx.x);
-    block_sum<1>(v, sh);
+    block_sum_f64<1>(v, sh);
     if (threadIdx.x == 0) prof[blockIdx.x] = v[0] / ((double)d.mx * d.my);
 }
 // the box's scaling and node kinds, and the patch rows' places

@@ -45,14 +45,33 @@ static __device__ __forceinline__ bool exchange(const Args& a, int& e, A (&v)[NV
     }
     __syncthreads();
     if (!xs.ok) return false;
-    A s[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) s[q] = threadIdx.x < G ? __ldcg(val + (size_t)q * G + threadIdx.x) : (A)0;
-    block_sum_t<A, NV>(s, sh);
     A* bc = (A*)xs.bc;
-    if (threadIdx.x == 0)
+    if constexpr (std::is_same<A, double>::value) {   // (a value per warp: the adds of FP64)
+        const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (q < NV) {
+            double s = 0.0;
+            for (unsigned g0 = 0; g0 < G; g0 += 160) {
+                double p[5];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) bc[q] = s[q];
+                for (int k = 0; k < 5; ++k) {
+                    const unsigned g = g0 + 32 * k + lane;
+                    p[k] = g < G ? __ldcg(val + (size_t)q * G + g) : 0.0;
+                }
+                s += ((p[0] + p[1]) + (p[2] + p[3])) + p[4];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) bc[q] = s;
+        }
+    } else {
+        A s[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) s[q] = threadIdx.x < G ? __ldcg(val + (size_t)q * G + threadIdx.x) : (A)0;
+        block_sum_t<A, NV>(s, sh);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) bc[q] = s[q];
+    }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < NV; ++q) tot[q] = bc[q];
