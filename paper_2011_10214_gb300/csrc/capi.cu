@@ -1140,7 +1140,7 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
     CUDA_OK(mark_stats(&cp, 1, c.stream));
     float ph[8] = {0};
     bool mixed = c.precision == PIFEPIC_MIXED;
-    // The host does not wait for each step: every step records its six phase
+    // The host does not wait for each step: every step records its phase
     // events into one of STEP_RING sets, and a set is read (after its last
     // event) only when it is reused and at the end, so the host keeps the
     // stream fed.  A photoemitting species' waiting list is watched with a
@@ -1165,15 +1165,19 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
         CUDA_OK(cudaStreamSynchronize(c.stream));
         return regrow_if_spilling(ctx, c.ph_species);
     };
-    std::vector<char> unread(STEP_RING, 0);
+    std::vector<char> unread(STEP_RING, 0), starts(STEP_RING, 0);   // starts: a step with a start event of its own
     auto read_set = [&](int slot) -> cudaError_t {
         cudaEvent_t* ev = &c.step_ev[6 * slot];
         cudaError_t e = cudaEventSynchronize(ev[5]);
         if (e != cudaSuccess) return e;
-        const int map[5] = {0, 1, 2, 3, 5};   // push, movers, inject, rebin, solve(+rhs+E)
-        for (int k = 0; k < 5; ++k) {
+        // a step that follows another at once starts at its end; the injection runs on the
+        // side stream, inside the time of the push and the movers
+        const cudaEvent_t at[5] = {starts[slot] ? ev[0] : c.step_ev[6 * ((slot + STEP_RING - 1) % STEP_RING) + 5],
+                                   ev[1], ev[2], ev[4], ev[5]};
+        const int map[4] = {0, 1, 3, 5};   // push, movers (and injection), rebin, solve(+rhs+E)
+        for (int k = 0; k < 4; ++k) {
             float t;
-            e = cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
+            e = cudaEventElapsedTime(&t, at[k], at[k + 1]);
             if (e != cudaSuccess) return e;
             ph[map[k]] += t;
         }
@@ -1182,10 +1186,14 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
     };
     for (int it = 0; it < nsteps; ++it) {
         if (it == FD_LOOK) CUDA_OK(settle_inside(c, it));
-        const int slot = it % STEP_RING;
+        // a set is read before it is reused, and before the end event of the step before it is
+        const int slot = it % STEP_RING, next = (it + 1) % STEP_RING;
         if (unread[slot]) CUDA_OK(read_set(slot));
+        if (unread[next]) CUDA_OK(read_set(next));
         cudaEvent_t* ev = &c.step_ev[6 * slot];
-        CUDA_OK(cudaEventRecord(ev[0], c.stream));
+        // (each event costs the stream some 2 us; a photoemitting step may follow a rebuild)
+        starts[slot] = it == 0 || it == FD_LOOK || each;
+        if (starts[slot]) CUDA_OK(cudaEventRecord(ev[0], c.stream));
         CUDA_OK(mixed ? launch_push_prep_mixed(c) : launch_push_prep(c));
         // the waiting list's push and the injection only append to the step's
         // mover list and add to the surface accumulators (atomics), so they run
@@ -1212,7 +1220,6 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
             CUDA_OK(e5);
         }
         CUDA_OK(cudaEventRecord(ev[2], c.stream));   // (the side stream's time beyond the push)
-        CUDA_OK(cudaEventRecord(ev[3], c.stream));
         CUDA_OK(mixed ? launch_rebin_mixed(c) : launch_rebin(c));
         CUDA_OK(cudaEventRecord(ev[4], c.stream));
         if (!c.external_E) CUDA_OK(run_solve(c));

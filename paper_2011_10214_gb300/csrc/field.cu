@@ -464,13 +464,21 @@ cudaError_t move_to_fd(Ctx& c) {
     return capture_pcg_graph(c);
 }
 
+// the solver's limits on the device: sent when they change (every solve writes the
+// rest of the state, and a copy per solve was 3 us of a step)
 static cudaError_t set_pcg_state(Ctx& c) {
+    const double lim[4] = {c.tol, (double)c.maxit, c.inner_red, c.inner_margin};
+    if (c.limits_sent && memcmp(lim, c.limits, sizeof(lim)) == 0) return cudaSuccess;
+    memcpy(c.limits, lim, sizeof(lim));
+    c.limits_sent = true;
     PcgState h = {};
     h.tol2 = c.tol * c.tol;
     h.maxit = c.maxit;
     h.inner_red2 = c.inner_red * c.inner_red;
     h.margin2 = c.inner_margin * c.inner_margin;
-    return cudaMemcpyAsync(c.scal, &h, sizeof(PcgState), cudaMemcpyHostToDevice, c.stream);
+    cudaError_t e = cudaMemcpyAsync(c.scal, &h, sizeof(PcgState), cudaMemcpyHostToDevice, c.stream);
+    if (e != cudaSuccess) c.limits_sent = false;
+    return e;
 }
 
 // whether the last solve met the tolerance (waits for the stream)

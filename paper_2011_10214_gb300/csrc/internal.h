@@ -226,6 +226,8 @@ struct Ctx {
     int maxit = 150;
     double inner_red = 1e-4;      // MIXED: inner solves stop at max(margin tol |b|, red |r0|)
     double inner_margin = 0.5;
+    bool limits_sent = false;     // the solver's limits are on the device as in limits
+    double limits[4] = {0, 0, 0, 0};
     int track = 0;
     int nbx = 0, nby = 0, nbz = 0, nblocks = 0;
     int bin_edge = BLK;           // particle bins of bin_edge^3 PIC cells (MIXED: 4 or 8; FP64: 4)
