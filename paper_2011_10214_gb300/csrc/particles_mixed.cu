@@ -325,8 +325,12 @@ PF_D void tile_flush19(const Launch& L, unsigned long long* W, const unsigned* W
 // A warp's next PUSH_DEPTH chunks are in flight at any time: one lane copies a chunk's 896
 // bytes into the warp's stage with a bulk copy (bins start on whole groups of 32 slots), so
 // the particles cost no address arithmetic and no registers while they travel.
-// HYBRID: the IFE mesh is finer than the PIC mesh, stayers deposit straight
-// onto its nodes (a separate instantiation keeps the common path's registers)
+// RF (instantiations of their own keep the common path's registers): 0, the IFE mesh is the PIC
+// mesh; 2, it is twice as fine and B = 4: stayers deposit into a tile of its 9^3 nodes, in the
+// 2^32 units a particle of the direct deposit (low and high halves, 8 copies a node, 47 KB), so
+// the sums are the same integers; 1, any finer mesh, whose tile has no room (17^3 nodes): eight
+// 64-bit atomics a particle straight onto its nodes.  4.1M particles in 32^3 cells of two IFE
+// cells a side: 189 us directly, 96 by the tile.
 constexpr int PUSH_DEPTH = 3;   // chunks in flight per warp
 constexpr int PUSH_CHUNKS = (BIN_MAX + 31) / 32;
 
@@ -335,12 +339,14 @@ constexpr int PUSH_CHUNKS = (BIN_MAX + 31) / 32;
 // stages' room later holds the masks' prefix counts and the list of slots to fill.
 // 16 deposit copies a node halve the atomics' bank conflicts against 8 (32, without any, were
 // no faster at 4,096 particles a bin and slower at 1,024); at B = 8 they would take 47 KB.
-template <int B, int NW>
+template <int RF, int B, int NW>
 struct PushSmem {
     static constexpr int TL = B + 1, TN = TL * TL * TL;
     static constexpr int NC = B == 4 ? 16 : 8;
     static constexpr size_t pp = sizeof(float4) * TN, pq = (pp + sizeof(float2) * TN + 127) / 128 * 128;
-    static constexpr size_t wt = (sizeof(unsigned) * NC * TN + 127) / 128 * 128;
+    static constexpr int TL2 = 2 * B + 1, TN2 = TL2 * TL2 * TL2;   // IFE nodes of a bin, refine 2
+    static constexpr int wn = RF == 2 ? 2 * 8 * TN2 : NC * TN;      // words of the deposit tile
+    static constexpr size_t wt = (sizeof(unsigned) * wn + 127) / 128 * 128;
     static constexpr size_t stg = sizeof(unsigned) * NW * PUSH_DEPTH * 7 * 32;
     static constexpr size_t mask = sizeof(unsigned) * PUSH_CHUNKS;
     static constexpr size_t bytes = pq + wt + stg + mask;
@@ -395,10 +401,10 @@ PF_D void bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long lo
                  : "memory");
 }
 
-template <bool HYBRID, int B, int NW>
-__global__ void __launch_bounds__(32 * NW, 32 / NW) k_push_bins_m(const __grid_constant__ Launch L, const __grid_constant__ ObjF of,
+template <int RF, int B, int NW>
+__global__ void __launch_bounds__(32 * NW, RF == 2 ? 3 : 32 / NW) k_push_bins_m(const __grid_constant__ Launch L, const __grid_constant__ ObjF of,
                                                      float dthf, const __grid_constant__ CUtensorMap tmE) {
-    using SM = PushSmem<B, NW>;
+    using SM = PushSmem<RF, B, NW>;
     constexpr int NT = 32 * NW;
     constexpr int TL = SM::TL, TN = SM::TN;
     extern __shared__ __align__(128) unsigned char push_smem[];
@@ -472,7 +478,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_push_bins_m(const __grid_c
             Eq[t] = make_float2(u.z, v.z);
         }
     __syncthreads();
-    for (int t = tid; t < SM::NC * TN; t += NT) Wt[t] = 0u;
+    for (int t = tid; t < SM::wn; t += NT) Wt[t] = 0u;
     __syncthreads();
     const float kf = (float)S.k;
     // the bin's cells inside the mesh, the reflecting faces it touches, and whether the
@@ -541,7 +547,16 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_push_bins_m(const __grid_c
             o[0] = (unsigned)(cell0 + ri + (rj << 11) + (rk << 22));
             o[32] = __float_as_uint(fx); o[64] = __float_as_uint(fy); o[96] = __float_as_uint(fz);
             o[128] = __float_as_uint(vx); o[160] = __float_as_uint(vy); o[192] = __float_as_uint(vz);
-            if (HYBRID) {          // hybrid grid: straight onto the IFE nodes
+            if (RF == 2) {         // hybrid grid, two IFE cells a cell
+                const float gx = 2.0f * fx, gy = 2.0f * fy, gz = 2.0f * fz, sx = floorf(gx), sy = floorf(gy),
+                            sz = floorf(gz);
+                const int t0 = 2 * ri + (int)sx + SM::TL2 * (2 * rj + (int)sy + SM::TL2 * (2 * rk + (int)sz));
+                long long Wf[8];
+                fixed_weights_f(weights_f(gx - sx, gy - sy, gz - sz), Wf);
+                const long long W7[7] = {Wf[0], Wf[1], Wf[2], Wf[3], Wf[4], Wf[5], Wf[6]};
+                int* lo = reinterpret_cast<int*>(Wt);
+                tile_deposit<long long, SM::TL2>(lo, lo + 8 * SM::TN2, 8 * t0 + (lane & 7), W7);
+            } else if (RF == 1) {  // finer: straight onto the IFE nodes
                 global_deposit_f(L, S.W, PF32{ri + x0, rj + y0, rk + z0, fx, fy, fz, vx, vy, vz});
             } else {               // (movers deposit in the rebin, with every mover of the step)
                 tile_deposit19<TL, SM::NC>(Wt, SM::NC * (ri + TL * (rj + TL * rk)) + copy, fx, fy, fz);
@@ -650,7 +665,22 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_push_bins_m(const __grid_c
         S.bstay[b] = total;
         sctr[C_PUSHED] = (unsigned)n;
     }
-    tile_flush19<TL, SM::NC>(L, S.W, Wt, x0, y0, z0);
+    if (RF == 2) {
+        const int* lo = reinterpret_cast<const int*>(Wt);
+        const int* hi = lo + 8 * SM::TN2;
+        for (int t = tid; t < SM::TN2; t += NT) {
+            long long v = 0;
+            for (int c = 0; c < 8; ++c) {
+                const int at = 8 * t + ((c + t) & 7);
+                v += tile_value(lo[at], hi[at]);
+            }
+            const int gi = 2 * x0 + t % SM::TL2, gj = 2 * y0 + t / SM::TL2 % SM::TL2, gk = 2 * z0 + t / (SM::TL2 * SM::TL2);
+            if (v && gi <= L.fmesh.nx && gj <= L.fmesh.ny && gk <= L.fmesh.nz)
+                atomicAdd(&S.W[node_id(L.fmesh, gi, gj, gk)], (unsigned long long)v);
+        }
+    } else if (RF == 0) {
+        tile_flush19<TL, SM::NC>(L, S.W, Wt, x0, y0, z0);
+    }
     __syncthreads();
     if (tid < NCTR && sctr[tid]) atomicAdd(&S.ctr[tid], (unsigned long long)sctr[tid]);
 }
@@ -959,15 +989,15 @@ __global__ void k_inject_counts(InjArgs a);   // particles.cu
 
 // one push launch; the kernel's dynamic shared-memory limit is raised once to what it
 // needs (above the 48 KB default)
-template <bool HYBRID, int B, int NW>
+template <int RF, int B, int NW>
 static cudaError_t push_bins_m(dim3 grid, cudaStream_t st, const Launch& L, const ObjF& of, float dthf,
                                const CUtensorMap& tm) {
-    using SM = PushSmem<B, NW>;
+    using SM = PushSmem<RF, B, NW>;
     static_assert(SM::bytes <= 200 * 1024, "push shared memory");
-    void* kern = (void*)k_push_bins_m<HYBRID, B, NW>;
+    void* kern = (void*)k_push_bins_m<RF, B, NW>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
     if (e != cudaSuccess) return e;
-    k_push_bins_m<HYBRID, B, NW><<<grid, 32 * NW, SM::bytes, st>>>(L, of, dthf, tm);
+    k_push_bins_m<RF, B, NW><<<grid, 32 * NW, SM::bytes, st>>>(L, of, dthf, tm);
     return cudaGetLastError();
 }
 // Warps per block by the slots of a bin (particles and a quarter more, of the fullest
@@ -981,8 +1011,8 @@ constexpr long long PUSH_SMALL = 3700, PUSH_LARGE = 6200;   // slots of a bin, a
 template <int B>
 static cudaError_t push_bins_by_fill(dim3 grid, cudaStream_t st, const Launch& L, const ObjF& of, float dthf,
                                      const CUtensorMap& tm, long long slots) {
-    if (slots < (B == 4 ? PUSH_SMALL : PUSH_LARGE)) return push_bins_m<false, B, B == 4 ? 4 : 8>(grid, st, L, of, dthf, tm);
-    return push_bins_m<false, B, B == 4 ? 8 : 16>(grid, st, L, of, dthf, tm);
+    if (slots < (B == 4 ? PUSH_SMALL : PUSH_LARGE)) return push_bins_m<0, B, B == 4 ? 4 : 8>(grid, st, L, of, dthf, tm);
+    return push_bins_m<0, B, B == 4 ? 8 : 16>(grid, st, L, of, dthf, tm);
 }
 
 // what precedes a push: the step's mover-list counts and node charges start at zero
@@ -1005,10 +1035,11 @@ cudaError_t launch_push_bins_mixed(Ctx& c) {
     cudaError_t e;
     if (c.bin_edge == 8)
         e = c.refine == 1 ? push_bins_by_fill<8>(grid, c.stream, L, of, dthf, c.tmapEf, slots)
-                          : push_bins_m<true, 8, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
+                          : push_bins_m<1, 8, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
     else
         e = c.refine == 1 ? push_bins_by_fill<4>(grid, c.stream, L, of, dthf, c.tmapEf, slots)
-                          : push_bins_m<true, 4, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
+                          : c.refine == 2 ? push_bins_m<2, 4, 8>(grid, c.stream, L, of, dthf, c.tmapEf)
+                                          : push_bins_m<1, 4, 8>(grid, c.stream, L, of, dthf, c.tmapEf);
     c.launches += 1;
     return e;
 }
