@@ -195,18 +195,18 @@ def cfg_desc(cfg, precision, extra=None):
 # GPU arm
 # ---------------------------------------------------------------------------------
 # FP64 push, from an ncu capture of one k_push_bins launch on the 32^3 sphere (4,076,523 particles):
-# sm__inst_executed_pipe_fp64.sum = 18,357,080 warp instructions (4.50 per particle, 144 lane operations),
-# DADD 183,285,395 + DMUL 256,496,282 + DFMA 9,065 thread instructions (107.9 flops per particle; the kernel
+# sm__inst_executed_pipe_fp64.sum = 12,559,933 warp instructions (3.08 per particle, 99 lane operations),
+# DADD 166,772,939 + DMUL 223,622,370 + DFMA 9,065 thread instructions (95.8 flops per particle; the kernel
 # keeps DADD and DMUL apart, no FMA contraction, for results bit-identical to the FP64 oracle)
-FP64_PIPE_WARP_INST_PER_PARTICLE = 18357080 / 4076523
-FP64_FLOPS_PER_PARTICLE_STEP = (183285395 + 256496282 + 2 * 9065) / 4076523
+FP64_PIPE_WARP_INST_PER_PARTICLE = 12559933 / 4076523
+FP64_FLOPS_PER_PARTICLE_STEP = (166772939 + 223622370 + 2 * 9065) / 4076523
 FP64_LANES_PER_CLK_SM = 2              # FP64 pipe: 2 lane operations per clock per SM (GB300)
 # PCG: 7 node-vector passes per iteration (p, x, r, z updates, the operator's read of p and write of q)
 SOLVE_BYTES_PER_NODE_ITER = {"mixed": 7 * 4, "fp64": 7 * 8}
 # DRAM bytes per pushed particle of one k_push_bins_m launch, from an ncu capture of the 64^3 sphere
 # bench workload (dram__bytes_read.sum + dram__bytes_write.sum over the launch's particles); None when
 # not measured for the current kernel
-PUSH_TRAFFIC_PER_PARTICLE = {"mixed": (930762240 + 860456448) / 32619866, "fp64": None}
+PUSH_TRAFFIC_PER_PARTICLE = {"mixed": (931127296 + 925939968) / 32619866, "fp64": None}
 NSM, DFMA_PER_CLK_SM = 152, 2          # GB300: 2 FP64 FMA per SM per clock
 
 
@@ -274,7 +274,7 @@ def roofline(precision, st, steps, ck):
                 "achieved": round(ach, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ach / peaks["hbm_gbs"], 4),
                 "traffic": None if tpp is None else round(tpp * per_launch),
-                "traffic_note": "ncu DRAM bytes per particle of a 64^3 sphere launch (54.9 B, 0.98 of the "
+                "traffic_note": "ncu DRAM bytes per particle of a 64^3 sphere launch (56.9 B, 1.02 of the "
                                 "algorithmic 56 B), scaled to this launch's particles",
                 "peak_source": src, "alg_bytes_per_launch": alg, "avg_launch_ms": push_ms}
     # bound by the FP64 pipe: its lane operations (every FP64-pipe warp instruction x 32 lanes: DADD, DMUL,

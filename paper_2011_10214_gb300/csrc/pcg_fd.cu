@@ -1,6 +1,8 @@
 // PCG of the MIXED field solve with a fast-diagonalisation preconditioner (Lynch,
-// Rice and Thomas 1964): the default for MIXED meshes of FD_MIN_NODES nodes or
-// more whose x-y plane fits in shared memory.  (Sec. 2.5: the matrix solve is a
+// Rice and Thomas 1964): in MIXED the default beyond the register-resident solver,
+// for single field solves of FD_MIN_NODES nodes or more, for contexts whose first
+// warm solve has settled and on batches' clusters, where the x-y plane fits in
+// shared memory.  (Sec. 2.5: the matrix solve is a
 // PCG iteration stopped on the relative residual; the paper names no
 // preconditioner.)
 //
@@ -30,8 +32,8 @@
 // only shapes the search directions -- the vectors, products with A, dot
 // products and the FP64 residual that ends the solve are not touched by the
 // split, and the iteration counts equal those of an FP32 transform.  (3xTF32
-// needs twice the products and splits in the inner loop: 1.5 against 0.5 us a
-// product here.)  A block takes one plane and a chunk of its output columns, so
+// needs twice the products and splits in the inner loop: 33 against 22 us an
+// iteration at 64^3, on the node layout.)  A block takes one plane and a chunk of its output columns, so
 // both products of a transform stay in the block: the plane split on its way into
 // shared memory, the first product's result split again next to it; the basis
 // matrices come split and in fragment order from L1 (16 bytes per lane).
@@ -47,8 +49,8 @@
 // nodes, absent neighbours (Dirichlet or beyond a Neumann face) read as zero, and a
 // row's coefficients depend on position only through the number of cubes on either
 // side (1 on a Neumann face, else 2).  On the node layout, one node at a time, the
-// passes issued about 830 instructions a node and iteration and ran at 20 us an
-// iteration at 64^3; they were bound by instruction issue.
+// passes issued about 830 instructions a node and iteration, bound by issue: 22 us
+// an iteration at 64^3, 18 in the box.
 //
 // One iteration is four team barriers, two of which carry the reductions
 // (Chronopoulos and Gear's form: both dot products after one matrix product):
