@@ -465,8 +465,9 @@ __global__ void k_inject(Launch L, InjArgs a) {
         int code = NONE, acc = -1;
         bool rejected = false;
         double p[3] = {0, 0, 0}, v[3] = {0, 0, 0};
+        InjSample sm;
+        if (__any_sync(0xffffffffu, mm < cnt)) sm = inject_sample(mm < cnt, d, mm, *a.step, s, L.mesh, L.dth);
         if (mm < cnt) {
-            InjSample sm = inject_sample(d, mm, *a.step, s, L.mesh, L.dth);
             double p0[3] = {sm.p0[0], sm.p0[1], sm.p0[2]};
             bool ok = sm.ok;
             for (int c = 0; c < 3; ++c) { p[c] = sm.p[c]; v[c] = sm.v[c]; }
@@ -900,9 +901,11 @@ __global__ void k_photo(Launch L, PhotoArgs a) {
         const long long m = base + threadIdx.x;
         bool emitted = false, alive = false, out = false;
         double p[3] = {0, 0, 0}, v[3] = {0, 0, 0};
+        double vn = 0.0;
+        const bool drawn = flux_normal(m < total, (unsigned long long)m, a.seed, key1, 0.0, vn);
         if (m < total) {
             const PhotoDev& d = a.tets[photo_tet_of(a.base, a.ne, m)];
-            const PhotoSample sm = photo_sample(d, (unsigned long long)m, a.seed, key1, a.vth, a.dth);
+            const PhotoSample sm = photo_sample(d, (unsigned long long)m, a.seed, key1, a.vth, a.dth, drawn, vn);
             for (int c = 0; c < 3; ++c) { p[c] = sm.p[c] * a.inv_r; v[c] = sm.v[c]; }   // to PIC units
             if (S.reflect) reflect_d(L.mesh, S.reflect, p[0], p[1], p[2], v[0], v[1], v[2]);
             emitted = sm.ok && !(level_set(L.obj, p[0], p[1], p[2]) < 0.0);

@@ -1090,9 +1090,11 @@ __global__ void k_photo_m(Launch L, PhotoArgs a) {
         const long long m = base + threadIdx.x;
         bool emitted = false, alive = false, out = false;
         PF32 p;
+        double vn = 0.0;
+        const bool drawn = flux_normal(m < total, (unsigned long long)m, a.seed, key1, 0.0, vn);
         if (m < total) {
             const PhotoDev& d = a.tets[photo_tet_of(a.base, a.ne, m)];
-            PhotoSample sm = photo_sample(d, (unsigned long long)m, a.seed, key1, a.vth, a.dth);
+            PhotoSample sm = photo_sample(d, (unsigned long long)m, a.seed, key1, a.vth, a.dth, drawn, vn);
             for (int c = 0; c < 3; ++c) sm.p[c] *= a.inv_r;   // IFE to PIC cell units (exact)
             if (S.reflect) reflect_d(L.mesh, S.reflect, sm.p[0], sm.p[1], sm.p[2], sm.v[0], sm.v[1], sm.v[2]);
             emitted = sm.ok && !(level_set(L.obj, sm.p[0], sm.p[1], sm.p[2]) < 0.0);

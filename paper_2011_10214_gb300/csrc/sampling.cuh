@@ -37,18 +37,47 @@ PF_D void box_muller(double u1, double u2, double& z0, double& z1) {
 }
 
 // flux-weighted normal speed (units of vth): proposal N(mu, 1), mu the mode of
-// v exp(-(v - s)^2 / 2), acceptance (v/mu) exp(1 - v/mu); bounded tries
-PF_D bool flux_normal(unsigned long long m, unsigned long long seed, unsigned long long key1, double s, double& v) {
-    double mu = 0.5 * (s + sqrt(s * s + 4.0));
-    for (int t = 0; t < MAX_TRIES; ++t) {
-        U64x4 r = philox4x64(m, 2 + t, 0, 0, seed, key1);
-        double z, z1;
-        box_muller(u01(r.v[0]), u01(r.v[1]), z, z1);
-        double vv = mu + z;
-        double ratio = vv / mu;
-        if (vv > 0.0 && u01(r.v[2]) < ratio * exp(1.0 - ratio)) { v = vv; return true; }
+// v exp(-(v - s)^2 / 2), acceptance (v/mu) exp(1 - v/mu); bounded tries, try t from
+// block 2 + t of counter m.  Called by whole warps (act: the lanes with a particle;
+// seed, key1 and s the same in all): a try is some 130 FP64 instructions, and two
+// thirds of them are accepted, so the lanes that are done take the next tries of
+// those that are not, and each particle takes its first accepted one -- the same
+// numbers in two rounds, where the slowest lane made four or five.
+PF_D bool flux_normal(bool act, unsigned long long m, unsigned long long seed, unsigned long long key1, double s, double& v) {
+    const double mu = 0.5 * (s + sqrt(s * s + 4.0));
+    const int lane = threadIdx.x & 31;
+    bool found = false;
+    int next = 0;                                  // this lane's particle's first try not made yet
+    for (;;) {
+        const unsigned pend = __ballot_sync(0xffffffffu, act && !found && next < MAX_TRIES);
+        if (!pend) return found;
+        // lane l takes try l % per of the pending particle number l / per
+        const int per = 32 / __popc(pend), nth = lane / per;
+        unsigned rest = pend;
+        for (int q = 0; q < nth; ++q) rest &= rest - 1;
+        const int owner = rest ? __ffs(rest) - 1 : lane;
+        const unsigned long long om = __shfl_sync(0xffffffffu, m, owner);
+        const int t = __shfl_sync(0xffffffffu, next, owner) + lane % per;
+        double vv = 0.0;
+        bool good = false;
+        if (rest && t < MAX_TRIES) {
+            U64x4 r = philox4x64(om, 2 + t, 0, 0, seed, key1);
+            double z, z1;
+            box_muller(u01(r.v[0]), u01(r.v[1]), z, z1);
+            vv = mu + z;
+            const double ratio = vv / mu;
+            good = vv > 0.0 && u01(r.v[2]) < ratio * exp(1.0 - ratio);
+        }
+        const unsigned hits = __ballot_sync(0xffffffffu, good);
+        const int at = per * __popc(pend & ((1u << lane) - 1));   // (of a pending lane: where its tries are)
+        const unsigned mine = ((pend >> lane) & 1) ? (hits >> at) & (per == 32 ? 0xffffffffu : (1u << per) - 1) : 0u;
+        const double got = __shfl_sync(0xffffffffu, vv, mine ? at + __ffs(mine) - 1 : lane);
+        if (mine) {
+            v = got;
+            found = true;
+        }
+        next += per;
     }
-    return false;
 }
 
 struct InjSample {
@@ -59,7 +88,8 @@ struct InjSample {
 // particle mm of stream d in step `step`: start point p0 on the face, velocity
 // v, position p after the partial first step; ok = false if every rejection
 // try failed.  Counter (mm, block, 0, 0), key (seed, purpose 2 | species | face | step).
-PF_D InjSample inject_sample(const InjectDev& d, int mm, long long step, int s, const Mesh& mesh, double dth) {
+// Called by whole warps (act: the lanes with a particle).
+PF_D InjSample inject_sample(bool act, const InjectDev& d, int mm, long long step, int s, const Mesh& mesh, double dth) {
     const int f = d.face, ax = f >> 1;
     const double sgn = (f & 1) ? -1.0 : 1.0;
     const int t1 = ax == 0 ? 1 : 0, t2 = ax == 2 ? 1 : 2;
@@ -70,7 +100,7 @@ PF_D InjSample inject_sample(const InjectDev& d, int mm, long long step, int s, 
     U64x4 b1 = philox4x64(m, 1, 0, 0, d.seed, key1);
     InjSample r;
     double vn = 0.0;
-    r.ok = flux_normal(m, d.seed, key1, sgn * d.drift[ax] / d.vth, vn);
+    r.ok = flux_normal(act, m, d.seed, key1, sgn * d.drift[ax] / d.vth, vn);
     double g1, g2;
     box_muller(u01(b1.v[0]), u01(b1.v[1]), g1, g2);
     r.p0[ax] = sgn > 0 ? 0.0 : nax[ax];
@@ -112,13 +142,13 @@ struct PhotoSample {
 // area, then sqrt(r1), r2), flux-weighted normal speed (zero drift), Gaussian
 // tangential speeds, then a fraction U of one step.  Blocks of counter (m, b):
 // 0 -> (triangle, r1, r2, U), 1 -> tangential normals, 2.. -> normal speed.
+// vn: the normal speed (flux_normal; ok: accepted).
 PF_D PhotoSample photo_sample(const PhotoDev& d, unsigned long long m, unsigned long long seed,
-                              unsigned long long key1, double vth, double dth) {
+                              unsigned long long key1, double vth, double dth, bool ok, double vn) {
     PhotoSample r;
+    r.ok = ok;
     U64x4 b0 = philox4x64(m, 0, 0, 0, seed, key1);
     U64x4 b1 = philox4x64(m, 1, 0, 0, seed, key1);
-    double vn = 0.0;
-    r.ok = flux_normal(m, seed, key1, 0.0, vn);
     double g1, g2;
     box_muller(u01(b1.v[0]), u01(b1.v[1]), g1, g2);
     const double ut = u01(b0.v[0]), r1 = u01(b0.v[1]), r2 = u01(b0.v[2]), U = u01(b0.v[3]);
