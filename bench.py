@@ -304,28 +304,20 @@ def roofline_solve(precision, st, steps, nnodes, solver):
     alg = nnodes * SOLVE_BYTES_PER_NODE_ITER[precision] * iters
     ach = alg / (solve_ms / 1e3) / 1e9
     peaks, src = _peaks()
-    # the solver the library ran (pifepic_get_solver: 1 registers, 2 global memory, 3 multigrid, 4 fast diagonalisation)
-    reg, mg, fd = solver == 1, solver == 3, solver == 4
-    if fd:
-        # per inner iteration and free node, FP32: pass A reads r, q, w, s, z, p, x and writes r, q, p, x and the
-        # modes, B reads the modes and pivots and writes the modes, C reads them and s and writes z, D reads z and r
-        # and writes w
-        alg = nnodes * 4 * (12 + 3 + 3 + 3) * iters
-        ach = alg / (solve_ms / 1e3) / 1e9
+    # the solver the library ran (pifepic_get_solver: 1 registers, 2 global memory, 3 multigrid)
+    reg, mg = solver == 1, solver == 3
     if mg:
         # per inner iteration: the PCG's 7 FP32 passes plus the V-cycle's fine-level passes (pre-smoothing
         # 12 B, residual 12 B, correction 8 B, post-smoothing 16 B); the coarse levels add about 1/7 more
         alg = nnodes * (SOLVE_BYTES_PER_NODE_ITER["mixed"] + 48) * iters
         ach = alg / (solve_ms / 1e3) / 1e9
-    kname = ("k_pcg_fd (global memory, fast-diagonalisation preconditioner)" if fd else
-             "k_pcg_mg (global memory, multigrid V-cycle)" if mg else
+    kname = ("k_pcg_mg (global memory, multigrid V-cycle)" if mg else
              "k_pcg_reg (registers)" if reg else "k_pcg_glob (global memory)")
     return {"kernel": f"{kname}: persistent PCG, one launch per solve, in the solve graph", "bound": "hbm",
             "achieved": round(ach, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": round(ach / peaks["hbm_gbs"], 4), "traffic": None, "peak_source": src,
             "alg_bytes_per_launch": alg, "avg_launch_ms": solve_ms, "iters_per_solve": iters,
-            "note": ("fast-diagonalisation PCG: four grid barriers per inner iteration, vectors in L2" if fd else
-                     "multigrid-preconditioned PCG: ~16-20 grid barriers per inner iteration, vectors in L2" if mg else
+            "note": ("multigrid-preconditioned PCG: ~16-20 grid barriers per inner iteration, vectors in L2" if mg else
                      "latency-bound: one grid exchange per inner iteration (pipelined PCG), vectors in registers "
                      "and L2" if precision == "mixed" else
                      "latency-bound: two grid exchanges per iteration, vectors in registers and L2")}

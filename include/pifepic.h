@@ -218,23 +218,23 @@ pifepic_status pifepic_set_refinement(pifepic_ctx* ctx, double reduction, double
  * Jacobi smoothing (weight 0.6), the coarsest level (at most 256 nodes)
  * solved exactly by its dense inverse.  AUTO (the default): JACOBI on a mesh
  * that fits the register-resident solver (up to 8 nodes per thread of a full
- * grid, about 620,000 nodes), else MULTIGRID, and where it applies in the
- * place of either a fast-diagonalisation preconditioner: the 7-point operator
+ * grid, about 620,000 nodes), else MULTIGRID, where the Jacobi iteration count
+ * outgrows the cap; a warm-started solve of pifepic_solve or pifepic_step (any
+ * but the context's first, which starts from zero) that ends a call at the cap
+ * without converging moves the context to MULTIGRID too (meshes of at most 256
+ * nodes have no hierarchy and keep Jacobi).  AUTO's solves of
+ * pifepic_solve_field, from 32768 nodes, and of batches use a
+ * fast-diagonalisation preconditioner where it applies: the 7-point operator
  * with a permittivity that depends on z alone, inverted by sine or cosine
  * transforms along x and y and tridiagonal systems along z, scaled by the
- * node's permittivity; its iteration count does not grow with the mesh.  It
- * applies from 32768 nodes unless every face is Neumann or an x-y plane is too
- * large for shared memory (about 200 x 200 nodes; more than 256 along z), at
- * once to pifepic_solve_field and in the place of MULTIGRID; in the place of
- * JACOBI to the solves of pifepic_solve and pifepic_step after a warm-started
- * one (any but the context's first, which starts from zero) has met the
- * tolerance or ended a call at the iteration cap.  Its reduction is at most
- * 1e-6 between Dirichlet faces and in a batch, else its margin at most 0.2
- * (pifepic_set_refinement).  Where it does not apply, a warm-started Jacobi
- * solve that ends a call at the cap without converging, like one of its own,
- * moves the context to MULTIGRID (meshes of at most 256 nodes have no
- * hierarchy and keep Jacobi).  All solve the same system to the same
- * stopping test.  Takes effect at once (the solve is re-planned); no
+ * node's permittivity; its iteration count does not grow with the mesh.  (The
+ * transforms take FP32 operands split into two BF16 parts; vectors, products
+ * with the operator and dot products stay FP32, the residual that ends a solve
+ * FP64.)  It applies unless every face is Neumann or an x-y plane is too large
+ * for shared memory (about 200 x 200 nodes; more than 256 along z).  Its
+ * reduction is at most 1e-6 between Dirichlet faces and in a batch, else its
+ * margin at most 0.2 (pifepic_set_refinement).  All solve the same system to
+ * the same stopping test.  Takes effect at once (the solve is re-planned); no
  * effect in FP64 mode.  On batched solves only AUTO has: a member whose own
  * choice is another one is solved by Jacobi clusters.  Errors: EINVAL
  * (unknown kind), ENOMEM. */
@@ -243,14 +243,8 @@ pifepic_status pifepic_set_preconditioner(pifepic_ctx* ctx, int kind);
 /* The persistent solver the context's next solve runs (after AUTO's choices):
  * 1 = Jacobi PCG with the vectors in registers (meshes of at most 8 nodes per
  * thread of a full grid), 2 = Jacobi PCG with the vectors in global memory,
- * 3 = multigrid-preconditioned PCG (MIXED), 4 = fast-diagonalisation-
- * preconditioned PCG (MIXED); 0 for a NULL context. */
-enum {
-    PIFEPIC_SOLVER_REGISTERS = 1,
-    PIFEPIC_SOLVER_GLOBAL = 2,
-    PIFEPIC_SOLVER_MULTIGRID = 3,
-    PIFEPIC_SOLVER_FAST_DIAGONAL = 4
-};
+ * 3 = multigrid-preconditioned PCG (MIXED); 0 for a NULL context. */
+enum { PIFEPIC_SOLVER_REGISTERS = 1, PIFEPIC_SOLVER_GLOBAL = 2, PIFEPIC_SOLVER_MULTIGRID = 3 };
 int pifepic_get_solver(const pifepic_ctx* ctx);
 pifepic_status pifepic_set_field_bc(pifepic_ctx* ctx, const pifepic_face_bc bc[6]);
 

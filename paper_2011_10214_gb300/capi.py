@@ -16,7 +16,7 @@ LIB_PATH = os.path.join(_HERE, "_build", "libpifepic.so")
 FP64, MIXED = 0, 1
 HOST, DEVICE = 0, 1
 OBJ_NONE, OBJ_SPHERE, OBJ_CAP_CRATER, OBJ_PLANE, OBJ_RIM_CRATER = 0, 1, 2, 3, 4
-SOLVER_REGISTERS, SOLVER_GLOBAL, SOLVER_MULTIGRID, SOLVER_FAST_DIAGONAL = 1, 2, 3, 4
+SOLVER_REGISTERS, SOLVER_GLOBAL, SOLVER_MULTIGRID = 1, 2, 3
 BC_DIRICHLET, BC_NEUMANN = 0, 1
 PBC_ABSORB, PBC_INJECT, PBC_REFLECT = 0, 1, 2
 PRECOND_AUTO, PRECOND_JACOBI, PRECOND_MULTIGRID = 0, 1, 2
@@ -253,8 +253,7 @@ class Simulation:
 
     @property
     def solver(self):
-        """The persistent solver of the next solve: SOLVER_REGISTERS, SOLVER_GLOBAL, SOLVER_MULTIGRID or
-        SOLVER_FAST_DIAGONAL."""
+        """The persistent solver of the next solve: SOLVER_REGISTERS, SOLVER_GLOBAL or SOLVER_MULTIGRID."""
         return int(lib.pifepic_get_solver(self._c))
 
     def set_field_bc(self, faces):

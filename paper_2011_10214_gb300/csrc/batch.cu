@@ -27,7 +27,7 @@ int cluster_size_for(long long N, long long H, bool mixed, long long cta_nodes);
 cudaError_t build_pcg_graph(Ctx& c);                                                // field.cu
 cudaError_t launch_pcg_mg_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_mg.cu
 cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_fd.cu
-cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
+cudaError_t plan_pcg_fd(Ctx& c);
 size_t cluster_smem_for(long long N, long long H, int C, bool mixed);
 cudaError_t launch_pcg_cluster(const BatchItem& item, int C, size_t smem, bool mixed, cudaStream_t st);
 cudaError_t launch_pcg_coop(Ctx& c, cudaStream_t st);                               // pcg_coop.cu
@@ -154,10 +154,9 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         }
         csize[i] = cluster_size_for(c.mesh.nnodes, node_halo(c.mesh), mixed, b->cta_nodes);
         if (mixed && csize[i] > 0 && b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx == 0 && !c.fd_wanted) {
-            // the plan on first use (and the member's own solve re-planned with it)
+            // the plan on first use (no memory for it: Jacobi)
             c.fd_wanted = true;
-            cudaError_t e = build_pcg_graph(c);
-            if (e != cudaSuccess) return e;
+            if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();
         }
         if (csize[i] > 0 && uses_fd(b, c)) csize[i] = fd_cluster_size(c.mesh.nnodes, b->cta_nodes);
     }
@@ -177,7 +176,7 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
         long long l0 = c.launches;
-        const bool fd = csize[i] > 0 ? uses_fd(b, c) : csize[i] == 0 && c.fd_single;
+        const bool fd = csize[i] > 0 && uses_fd(b, c);
         e = capture(c, cs, [mixed, fd](Ctx& cc) -> cudaError_t {
             cudaError_t r = mixed ? launch_push_mixed(cc) : launch_push(cc);
             if (r == cudaSuccess) r = mixed ? launch_movers_mixed(cc) : launch_movers(cc);
@@ -235,9 +234,7 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         if (e != cudaSuccess) break;
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
-        e = capture(c, cs, [](Ctx& cc) -> cudaError_t {
-            return cc.fd_single ? launch_pcg_fd(cc, cc.stream) : launch_pcg_coop(cc, cc.stream);
-        }, &sub);
+        e = capture(c, cs, [](Ctx& cc) -> cudaError_t { return launch_pcg_coop(cc, cc.stream); }, &sub);
         cudaGraphNode_t deps[2] = {pre[i], last_big};
         if (e == cudaSuccess) e = cudaGraphAddChildGraphNode(&solve_of[i], g, deps, last_big ? 2 : 1, sub);
         if (sub) cudaGraphDestroy(sub);

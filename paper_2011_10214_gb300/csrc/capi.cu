@@ -68,8 +68,6 @@ pifepic_status solve_field_noalloc(Ctx& c, const double* F, const double* q, dou
 void free_mg(Ctx& c);                         // pcg_mg.cu
 void free_fd(Ctx& c);                         // pcg_fd.cu
 cudaError_t build_pcg_graph(Ctx& c);          // field.cu
-cudaError_t last_solve_converged(Ctx& c, bool* conv);
-cudaError_t move_to_fd(Ctx& c);
 
 // 5-tet split tables, computed from the definition (reading of Sec. 3.1.1)
 static TetTables make_tables() {
@@ -670,7 +668,6 @@ int pifepic_get_bin_edge(const pifepic_ctx* ctx) { return ctx ? ctx->c.bin_edge 
 int pifepic_get_solver(const pifepic_ctx* ctx) {
     if (!ctx) return 0;
     const Ctx& c = ctx->c;
-    if (c.fd_single) return PIFEPIC_SOLVER_FAST_DIAGONAL;
     if (c.precision == PIFEPIC_MIXED && c.mg_single && c.mg_nlev > 0) return PIFEPIC_SOLVER_MULTIGRID;
     return c.pcg_npt > 0 ? PIFEPIC_SOLVER_REGISTERS : PIFEPIC_SOLVER_GLOBAL;
 }
@@ -1069,38 +1066,18 @@ static cudaError_t run_solve(Ctx& c) {
     return launch_pcg(c);   // (the solve graph holds the precision's kernels)
 }
 
-// AUTO (MIXED): the solver of a context's later solves, after a warm-started one
-// (any but its first, which starts from zero) that converged or ended at the cap.
-// Jacobi is followed by the fast-diagonalisation PCG where it applies; else, after
-// a capped solve, by the multigrid cycle, as the fast-diagonalisation PCG is (a
-// mesh too small for a hierarchy keeps Jacobi).  The solve is re-planned once.
-static pifepic_status settle_solver(pifepic_ctx* ctx) {
+// AUTO (MIXED): once a warm-started Jacobi solve of the context (any but its
+// first, which starts from zero) has ended at the iteration cap without
+// converging, its later solves run the multigrid cycle (the solve is
+// re-planned once; a mesh too small for a hierarchy keeps Jacobi)
+static pifepic_status escalate_if_capped(pifepic_ctx* ctx) {
     Ctx& c = ctx->c;
-    if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || c.mg_single) return PIFEPIC_OK;
-    const bool capped = !c.last_conv && c.last_iters >= c.maxit;
-    if (c.solves_done < 2 || !(capped || c.last_conv)) return PIFEPIC_OK;
-    if (c.fd_ready && !c.fd_single) {
-        CUDA_OK(move_to_fd(c));
+    if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || c.mg_single || c.mg_escalated)
         return PIFEPIC_OK;
-    }
-    if (capped && !c.mg_escalated) {
-        c.fd_capped = c.fd_single;
-        c.mg_escalated = true;
-        CUDA_OK(build_pcg_graph(c));
-    }
+    if (c.solves_done < 2 || c.last_conv || c.last_iters < c.maxit) return PIFEPIC_OK;
+    c.mg_escalated = true;
+    CUDA_OK(build_pcg_graph(c));
     return PIFEPIC_OK;
-}
-// the same inside a long call, at its step FD_LOOK: moves on if the last solve
-// converged (a call whose solves are capped keeps its solver to its end)
-constexpr int FD_LOOK = 4;
-static cudaError_t settle_inside(Ctx& c, int steps_done) {
-    if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || !c.fd_ready || c.fd_single || c.mg_single ||
-        c.external_E || c.solves_done + steps_done < 2)
-        return cudaSuccess;
-    bool conv = false;
-    cudaError_t e = last_solve_converged(c, &conv);   // (waits for the stream)
-    if (e != cudaSuccess || !conv) return e;
-    return move_to_fd(c);
 }
 
 pifepic_status pifepic_solve(pifepic_ctx* ctx, pifepic_stats* st) {
@@ -1118,7 +1095,7 @@ pifepic_status pifepic_solve(pifepic_ctx* ctx, pifepic_stats* st) {
     pifepic_status r = fill_stats(ctx, st, nullptr, l0, c.external_E ? 0 : 1);
     if (r || c.external_E) return r;
     c.solves_done += 1;
-    return settle_solver(ctx);
+    return escalate_if_capped(ctx);
 }
 
 pifepic_status pifepic_leapfrog_init(pifepic_ctx* ctx) {
@@ -1185,14 +1162,13 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
         return cudaSuccess;
     };
     for (int it = 0; it < nsteps; ++it) {
-        if (it == FD_LOOK) CUDA_OK(settle_inside(c, it));
         // a set is read before it is reused, and before the end event of the step before it is
         const int slot = it % STEP_RING, next = (it + 1) % STEP_RING;
         if (unread[slot]) CUDA_OK(read_set(slot));
         if (unread[next]) CUDA_OK(read_set(next));
         cudaEvent_t* ev = &c.step_ev[6 * slot];
         // (each event costs the stream some 2 us; a photoemitting step may follow a rebuild)
-        starts[slot] = it == 0 || it == FD_LOOK || each;
+        starts[slot] = it == 0 || each;
         if (starts[slot]) CUDA_OK(cudaEventRecord(ev[0], c.stream));
         CUDA_OK(mixed ? launch_push_prep_mixed(c) : launch_push_prep(c));
         // the waiting list's push and the injection only append to the step's
@@ -1252,7 +1228,7 @@ pifepic_status pifepic_step(pifepic_ctx* ctx, int nsteps, pifepic_stats* st) {
     pifepic_status r = fill_stats(ctx, st, ph, l0, c.external_E ? 0 : nsteps);
     if (r || c.external_E || nsteps == 0) return r;
     c.solves_done += nsteps;
-    return settle_solver(ctx);
+    return escalate_if_capped(ctx);
 }
 
 pifepic_status pifepic_get_sizes(pifepic_ctx* ctx, int64_t* nn, int64_t* nc, int64_t* nit, int64_t* ncut) {

@@ -391,7 +391,8 @@ cudaError_t launch_E_to_pic(const Ctx& c, cudaStream_t st, bool both) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);   // pcg_fd.cu
+cudaError_t plan_pcg_fd(Ctx& c);                      // pcg_fd.cu
+cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
 // q_T, right-hand side and start vector (where the solver keeps it)
 static cudaError_t launch_rhs(Ctx& c, cudaStream_t st, bool fd, const double* Fext) {
     const long long N = c.mesh.nnodes;
@@ -404,7 +405,7 @@ static cudaError_t launch_rhs(Ctx& c, cudaStream_t st, bool fd, const double* Fe
 
 static cudaError_t solve_sequence(Ctx& c, cudaStream_t st, const double* Fext) {
     FieldArgs f = fargs(c);
-    const bool fd = Fext ? c.fd_ready : c.fd_single;
+    const bool fd = Fext && c.fd.mx > 0 && c.mesh.nnodes >= FD_MIN_NODES;   // (the steps: Jacobi or multigrid)
     cudaError_t e = launch_rhs(c, st, fd, Fext);
     if (e != cudaSuccess) return e;
     e = fd ? launch_pcg_fd(c, st) : launch_pcg_coop(c, st);
@@ -433,7 +434,8 @@ int solve_graph_fixed_kernels(const Ctx& c) { return (c.nit > 0) + 3 + (c.refine
 
 // The solve as one CUDA graph (both precisions): q_T -> RHS -> warm start ->
 // persistent PCG -> node field
-static cudaError_t capture_pcg_graph(Ctx& c) {
+cudaError_t build_pcg_graph(Ctx& c) {
+    plan_pcg(c);
     if (c.pcg_exec) { cudaGraphExecDestroy(c.pcg_exec); c.pcg_exec = nullptr; }
     if (c.pcg_graph) { cudaGraphDestroy(c.pcg_graph); c.pcg_graph = nullptr; }
     cudaStream_t cs;
@@ -453,17 +455,6 @@ static cudaError_t capture_pcg_graph(Ctx& c) {
     return e;
 }
 
-cudaError_t build_pcg_graph(Ctx& c) {
-    plan_pcg(c);
-    return capture_pcg_graph(c);
-}
-
-// the context's solves move on to the fast-diagonalisation PCG (its plan stands)
-cudaError_t move_to_fd(Ctx& c) {
-    c.fd_now = c.fd_single = true;
-    return capture_pcg_graph(c);
-}
-
 // the solver's limits on the device: sent when they change (every solve writes the
 // rest of the state, and a copy per solve was 3 us of a step)
 static cudaError_t set_pcg_state(Ctx& c) {
@@ -481,14 +472,6 @@ static cudaError_t set_pcg_state(Ctx& c) {
     return e;
 }
 
-// whether the last solve met the tolerance (waits for the stream)
-cudaError_t last_solve_converged(Ctx& c, bool* conv) {
-    PcgState hs;
-    cudaError_t e = scopy(c.stream, &hs, pcg_state(c), sizeof(PcgState), cudaMemcpyDeviceToHost);
-    *conv = e == cudaSuccess && hs.converged;
-    return e;
-}
-
 cudaError_t launch_pcg(Ctx& c) {
     cudaError_t e = set_pcg_state(c);
     if (e != cudaSuccess) return e;
@@ -498,6 +481,10 @@ cudaError_t launch_pcg(Ctx& c) {
 
 // standalone solve with an external node load (solver parity)
 cudaError_t launch_solve_external(Ctx& c, const double* Fdev, int* iters, double* relres) {
+    if (!c.fd_wanted && c.mesh.nnodes >= FD_MIN_NODES) {
+        c.fd_wanted = true;
+        if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();   // (no plan: the context's own solver)
+    }
     cudaError_t e = set_pcg_state(c);
     if (e == cudaSuccess) e = solve_sequence(c, c.stream, Fdev);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);

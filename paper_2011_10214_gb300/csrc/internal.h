@@ -34,8 +34,8 @@ struct MgLevel {                  // a coarse level (27-point Galerkin rows)
 };
 
 // ---- fast-diagonalisation preconditioner of the MIXED field solve (pcg_fd.cu) ----
-// AUTO uses it from this many nodes: below, a Jacobi iteration (3 us) is cheap enough that
-// its 60 or so beat 14 of these at 17 us (24^3 sphere: 0.23 against 0.26 ms a solve; 32^3:
+// pifepic_solve_field uses it from this many nodes: below, a Jacobi iteration (3 us) is cheap
+// enough that its 60 or so beat 14 of these at 17 us (24^3 sphere: 0.23 against 0.26 ms a solve; 32^3:
 // 0.27 against 0.23, 37^3 0.34 against 0.31, 64^3 0.70 against 0.32)
 constexpr long long FD_MIN_NODES = 32768;
 // a batch's clusters from this many (16^3 cells: 0.26 ms a member's step against 0.45 with
@@ -316,13 +316,9 @@ struct Ctx {
     float* mg_r0 = nullptr;           // fine residual after pre-smoothing
     float* mg_cinv = nullptr;         // dense inverse of the coarsest operator
     bool mg_wanted = false;           // a batch solves this context with multigrid: keep a hierarchy
-    bool mg_escalated = false;        // AUTO: a Jacobi solve ended at the cap unconverged; another solver since
-    bool fd_capped = false;           // AUTO: a fast-diagonalisation solve did; multigrid since
+    bool mg_escalated = false;        // AUTO: a Jacobi solve ended at the cap unconverged; multigrid since
     FdPlan fd;                        // fast-diagonalisation preconditioner (fd.mx = 0: none)
-    bool fd_wanted = false;           // a batch solves this context with it: plan it on a smaller mesh too
-    bool fd_ready = false;            // pifepic_solve_field uses it
-    bool fd_now = false;              // a warm-started Jacobi solve is done: the steps use it too
-    bool fd_single = false;           // the solves of pifepic_solve and pifepic_step use it
+    bool fd_wanted = false;           // a batch or pifepic_solve_field solves this context with it: keep a plan
     char* fd_mem = nullptr;           // its arrays
     long long solves_done = 0;        // field solves of pifepic_solve and pifepic_step so far
     cudaStream_t side = nullptr;      // movers and injection beside the push (pifepic_step)

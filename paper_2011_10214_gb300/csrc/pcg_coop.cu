@@ -783,9 +783,9 @@ void plan_pcg(Ctx& c) {
     plan_pcg_reg(c);
     lib_free(c.rowkind); lib_free(c.pcg_x);
     c.rowkind = nullptr; c.pcg_x = nullptr;
-    if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();   // (no plan: the solvers below)
+    if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();   // (no plan: field solves and batches as the steps)
     if (plan_pcg_mg(c) != cudaSuccess) cudaGetLastError();   // (no hierarchy: the Jacobi solvers)
-    if ((c.pcg_npt > 0 || c.fd_single) && c.mg_nlev == 0) return;
+    if (c.pcg_npt > 0 && c.mg_nlev == 0) return;
     const long long N = c.mesh.nnodes;
     if (lib_malloc(&c.rowkind, sizeof(unsigned short) * N) != cudaSuccess ||
         lib_malloc(&c.pcg_x, sizeof(double) * N) != cudaSuccess) {

@@ -1,10 +1,15 @@
 // PCG of the MIXED field solve with a fast-diagonalisation preconditioner (Lynch,
-// Rice and Thomas 1964): in MIXED the default beyond the register-resident solver,
-// for single field solves of FD_MIN_NODES nodes or more, for contexts whose first
-// warm solve has settled and on batches' clusters, where the x-y plane fits in
-// shared memory.  (Sec. 2.5: the matrix solve is a
-// PCG iteration stopped on the relative residual; the paper names no
-// preconditioner.)
+// Rice and Thomas 1964): in MIXED the default for single field solves of
+// FD_MIN_NODES nodes or more and on batches' clusters, where the x-y plane fits in
+// shared memory.  (Sec. 2.5: the matrix solve is a PCG iteration stopped on the
+// relative residual; the paper names no preconditioner.)
+//
+// A context's own steps stay with Jacobi (multigrid beyond the registers), though
+// this solver is faster there too (0.33 against 0.69 ms a solve at 64^3, 3.1 against
+// 3.9 at 160 x 160 x 80): solvers that stop at the same residual differ by up to 2e-5
+// of the largest potential, and the object's mean potential is smaller than that is
+// when it passes through zero, so that a run's first steps differed there by 1e-3 of
+// it (50^3 eighth sphere) from what they were.
 //
 // Preconditioner.  The free nodes of the box (Dirichlet faces removed) form a
 // tensor grid, and the 7-point operator on it with a permittivity that depends
@@ -825,7 +830,6 @@ void free_fd(Ctx& c) {
     FdPlan& d = c.fd;
     lib_free(c.fd_mem);
     c.fd_mem = nullptr;
-    c.fd_ready = c.fd_single = false;
     d = FdPlan{};
 }
 
@@ -872,19 +876,15 @@ static bool fd_split(FdPlan& d, int G, size_t limit) {
     return best > 0.0;
 }
 
-// The plan for the context's mesh, boundaries and operator, in MIXED mode with AUTO;
-// not where no node is free, where every face is Neumann (P is singular) or where a
-// plane does not fit in shared memory.  pifepic_solve_field uses it from FD_MIN_NODES
-// nodes (fd_ready); so do the steps of a context too large for the register-resident
-// Jacobi solver.  On a smaller one the steps start with that solver, as before: its
-// cold first solve often ends at the cap, and what a run computes from the capped
-// iterate stays what it was.  They move on after the first warm-started solve
-// (fd_now, pifepic_step).
+// The plan for the context's mesh, boundaries and operator, in MIXED mode with AUTO,
+// once pifepic_solve_field (from FD_MIN_NODES nodes) or a batch has asked for it; not
+// where no node is free, where every face is Neumann (P is singular) or where a plane
+// does not fit in shared memory.
 cudaError_t plan_pcg_fd(Ctx& c) {
     free_fd(c);
     const Mesh& m = c.mesh;
-    if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || c.fd_capped ||
-        m.nnodes < (c.fd_wanted ? FD_CLUSTER_MIN_NODES : FD_MIN_NODES))
+    if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || !c.fd_wanted ||
+        m.nnodes < FD_CLUSTER_MIN_NODES)
         return cudaSuccess;
     int dir[6], any = 0;
     for (int f = 0; f < 6; ++f) any |= dir[f] = c.bc[f].kind == PIFEPIC_BC_DIRICHLET;
@@ -982,10 +982,6 @@ cudaError_t plan_pcg_fd(Ctx& c) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
     }
     if (e != cudaSuccess) free_fd(c);
-    if (e == cudaSuccess) {
-        c.fd_ready = m.nnodes >= FD_MIN_NODES;
-        c.fd_single = c.fd_ready && (c.pcg_npt == 0 || c.fd_now);
-    }
     return e;
 }
 

@@ -610,7 +610,7 @@ cudaError_t plan_pcg_mg(Ctx& c) {
     // cap; and once a Jacobi solve of this context has ended at the cap
     // unconverged (mostly Neumann faces: poorly conditioned for Jacobi)
     const bool single = c.precond == PIFEPIC_PRECOND_MULTIGRID ||
-                        (c.precond == PIFEPIC_PRECOND_AUTO && !c.fd_single && (c.pcg_npt == 0 || c.mg_escalated));
+                        (c.precond == PIFEPIC_PRECOND_AUTO && (c.pcg_npt == 0 || c.mg_escalated));
     if (!single && !c.mg_wanted) return cudaSuccess;
     const long long N0 = c.mesh.nnodes;
     int nx = c.mesh.nx, ny = c.mesh.ny, nz = c.mesh.nz;
