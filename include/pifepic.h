@@ -400,7 +400,9 @@ pifepic_status pifepic_solve_field(pifepic_ctx* ctx, const double* F, const doub
  * must share one precision; their own streams are synchronised before the
  * batch stream (given at creation) takes over.  A member's results do not
  * depend on the other members.  The graph is rebuilt on the next step after
- * add / remove / set_cta_nodes.  stats (if not NULL) receives one entry per
+ * add / remove / set_cta_nodes / set_preconditioner, and after a member's own
+ * solve was re-planned (its pifepic_set_preconditioner, or a solve of its own
+ * that ended at the cap).  stats (if not NULL) receives one entry per
  * member, in member order.  The batch borrows the contexts: destroy the batch
  * first. */
 typedef struct pifepic_batch pifepic_batch;

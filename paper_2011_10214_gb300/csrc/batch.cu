@@ -90,6 +90,7 @@ struct pifepic_batch {
     int cta_nodes = 8192;
     int precond = PIFEPIC_PRECOND_AUTO;   // MIXED members: MULTIGRID = multigrid clusters, else Jacobi clusters
     bool dirty = true;
+    std::vector<unsigned long long> plan_gen;   // the members' Ctx::plan_gen when the graph was built
     std::vector<long long> kernels;   // kernels per step of each instance (its share of the batch graph)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -160,6 +161,8 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         }
         if (csize[i] > 0 && uses_fd(b, c)) csize[i] = fd_cluster_size(c.mesh.nnodes, b->cta_nodes);
     }
+    b->plan_gen.resize(n);
+    for (int i = 0; i < n; ++i) b->plan_gen[i] = b->ctx[i]->c.plan_gen;
     const int groups[6] = {16, 8, 4, 2, 1, 0};
     std::vector<int> order;
     for (int g : groups)
@@ -313,6 +316,9 @@ pifepic_status pifepic_batch_step(pifepic_batch* b, int nsteps, pifepic_stats* s
         cudaError_t e = cudaStreamSynchronize(x->c.stream);
         if (e != cudaSuccess) return batch_fail(b, PIFEPIC_ECUDA, cudaGetErrorString(e));
     }
+    // a member's solve may have been re-planned since (pifepic_set_preconditioner, a solve of its
+    // own that ended at the cap, another batch): the graph's copies of its pointers are void
+    for (size_t i = 0; i < b->ctx.size() && !b->dirty; ++i) b->dirty = b->plan_gen[i] != b->ctx[i]->c.plan_gen;
     if (b->dirty) {
         cudaError_t e = build_batch_graph(b);
         if (e != cudaSuccess) return batch_fail(b, PIFEPIC_ECUDA, std::string("batch graph: ") + cudaGetErrorString(e));

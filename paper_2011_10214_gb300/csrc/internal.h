@@ -320,6 +320,9 @@ struct Ctx {
     FdPlan fd;                        // fast-diagonalisation preconditioner (fd.mx = 0: none)
     bool fd_wanted = false;           // a batch or pifepic_solve_field solves this context with it: keep a plan
     char* fd_mem = nullptr;           // its arrays
+    // plans made so far (plan_pcg): each frees the arrays of the one before, which a batch's
+    // graph may hold
+    unsigned long long plan_gen = 0;
     long long solves_done = 0;        // field solves of pifepic_solve and pifepic_step so far
     cudaStream_t side = nullptr;      // movers and injection beside the push (pifepic_step)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

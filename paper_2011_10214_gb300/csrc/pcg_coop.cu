@@ -775,6 +775,7 @@ cudaError_t plan_pcg_mg(Ctx& c);   // pcg_mg.cu: the multigrid hierarchy (MIXED)
 cudaError_t plan_pcg_fd(Ctx& c);   // pcg_fd.cu: the fast-diagonalisation preconditioner (MIXED), if selected
 
 void plan_pcg(Ctx& c) {
+    c.plan_gen += 1;
     // the exchanges count arrivals in multiples of their grid size, which differs
     // between the solvers: a new plan starts the counters (and the pipelined
     // loop's fallback flag) afresh

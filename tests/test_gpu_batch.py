@@ -150,3 +150,51 @@ def test_cluster_solves_match_single_instance_solves(precision, precond):
     b.close()
     for s in sims:
         s.close()
+
+
+@pytest.mark.parametrize("precond", ["auto", "multigrid"])
+def test_replanned_members_rebuild_the_graph(precond):
+    """A member's solve re-planned between two batched steps -- its preconditioner set, its own
+    solve ended at the cap, another batch's wish -- frees arrays that the graph was captured
+    with: the next step rebuilds it, and steps as a fresh batch does (to the bit)."""
+    from paper_2011_10214_gb300 import capi
+
+    def run(fresh):
+        sims = [_member(MEMBERS[1], capi.MIXED), _member(MEMBERS[2], capi.MIXED),
+                capi.from_config(MEMBERS[1], precision=capi.MIXED, pcg_max_iter=4)]
+        out, batch = [], None
+
+        def step():
+            nonlocal batch
+            if fresh and batch is not None:
+                batch.close()
+            if fresh or batch is None:
+                batch = capi.Batch(sims)
+                if precond == "multigrid":
+                    batch.set_preconditioner(capi.PRECOND_MULTIGRID)
+            st = batch.step(1)
+            out.append([(s.potential(), s.node_charge(0), t["pcg_iters"]) for s, t in zip(sims, st)])
+        step()
+        sims[0].set_preconditioner(capi.PRECOND_JACOBI)
+        step()
+        sims[0].set_preconditioner(capi.PRECOND_AUTO)
+        step()
+        for _ in range(2):                       # the second, warm-started, escalates
+            assert sims[2].solve()["pcg_converged"] == 0
+        assert sims[2].solver == capi.SOLVER_MULTIGRID
+        step()
+        other = capi.Batch([sims[1]])            # plans the member for itself
+        other.set_preconditioner(capi.PRECOND_MULTIGRID if precond == "auto" else capi.PRECOND_AUTO)
+        other.step(1)
+        step()
+        other.close()
+        batch.close()
+        for s in sims:
+            s.close()
+        return out
+    kept, new = run(False), run(True)
+    for k, (a, b) in enumerate(zip(kept, new)):
+        for (phi, W, it), (phi2, W2, it2) in zip(a, b):
+            assert np.array_equal(phi, phi2) and np.array_equal(W, W2) and it == it2, k
+    if precond == "auto":                        # the member's choice took effect at once, and back
+        assert kept[1][0][2] > 2 * kept[0][0][2] and kept[2][0][2] < 0.5 * kept[1][0][2]
