@@ -26,7 +26,8 @@ pifepic_status finish_stats(pifepic_ctx* ctx, long long kernels, pifepic_stats* 
 int cluster_size_for(long long N, long long H, bool mixed, long long cta_nodes);   // pcg_cluster.cu
 cudaError_t build_pcg_graph(Ctx& c);                                                // field.cu
 cudaError_t launch_pcg_mg_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_mg.cu
-cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_fd.cu
+int fd_cluster_size(const Ctx& c, long long cta_nodes);                             // pcg_fd.cu
+cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st);
 cudaError_t plan_pcg_fd(Ctx& c);
 size_t cluster_smem_for(long long N, long long H, int C, bool mixed);
 cudaError_t launch_pcg_cluster(const BatchItem& item, int C, size_t smem, bool mixed, cudaStream_t st);
@@ -40,7 +41,11 @@ cudaError_t launch_movers_mixed(Ctx& c);
 cudaError_t launch_inject_mixed(Ctx& c);
 cudaError_t launch_rebin_mixed(Ctx& c);
 
-constexpr long long FD_CTA_SHARE = 4;   // fast-diagonalisation clusters: cta_nodes / 4 nodes per CTA at most
+// Fast-diagonalisation clusters: cta_nodes / 4 nodes per CTA at most.  An iteration is
+// a few passes over the nodes between barriers of 0.3 us, with the planes' transforms
+// in the middle, so more CTAs pay longer than for the Jacobi clusters, whose whole
+// working set only has to fit.
+constexpr long long FD_CTA_SHARE = 4;
 constexpr double CL_INNER_RED = 1e-6;   // the batched Jacobi clusters' inner reduction (at most)
 
 static BatchItem make_item(Ctx& c) {
@@ -105,21 +110,6 @@ static pifepic_status batch_fail(pifepic_batch* b, pifepic_status st, const std:
 
 static long long node_halo(const Mesh& m) { return (long long)m.NX * m.NY + m.NX + 1; }
 
-// a member's cluster solves with the fast-diagonalisation preconditioner
-static bool uses_fd(const pifepic_batch* b, const Ctx& c) {
-    return b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx > 0;
-}
-
-// Its cluster: the smallest that keeps each CTA at or under a quarter of cta_nodes.  An
-// iteration is a few passes over the nodes between barriers of 0.3 us, with the
-// planes' transforms in the middle, so more CTAs pay longer than for the Jacobi
-// clusters, whose whole working set only has to fit.
-static int fd_cluster_size(long long N, long long cta_nodes) {
-    int C = 1;
-    while (C < 16 && (N + C - 1) / C > cta_nodes / FD_CTA_SHARE) C *= 2;
-    return C;
-}
-
 // The batch step as one graph: per instance a chain of its particle phases,
 // right-hand side, field solve (one cluster launch; an instance too large for
 // a cluster uses the single-instance persistent solver) and node field, so
@@ -133,8 +123,10 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
     // the solve of each instance: csize = its Jacobi cluster size (0: too large
     // for a cluster, the single-instance persistent solver); members solved by
     // the multigrid cluster kernel (MIXED, with a hierarchy) get csize -2 and
-    // their cluster size in mg_c
+    // their cluster size in mg_c, those by the fast-diagonalisation one its
+    // cluster size in csize and a mark in fd
     std::vector<int> csize(n, -1), mg_c(n, 0);
+    std::vector<char> fd(n, 0);
     std::vector<int> mg_members;
     for (int i = 0; i < n; ++i) {
         Ctx& c = b->ctx[i]->c;
@@ -159,7 +151,10 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             c.fd_wanted = true;
             if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();
         }
-        if (csize[i] > 0 && uses_fd(b, c)) csize[i] = fd_cluster_size(c.mesh.nnodes, b->cta_nodes);
+        if (csize[i] > 0 && b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx > 0) {
+            const int C = fd_cluster_size(c, b->cta_nodes / FD_CTA_SHARE);
+            if (C > 0) { csize[i] = C; fd[i] = 1; }
+        }
     }
     b->plan_gen.resize(n);
     for (int i = 0; i < n; ++i) b->plan_gen[i] = b->ctx[i]->c.plan_gen;
@@ -179,13 +174,13 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
         long long l0 = c.launches;
-        const bool fd = csize[i] > 0 && uses_fd(b, c);
-        e = capture(c, cs, [mixed, fd](Ctx& cc) -> cudaError_t {
+        const bool boxed = fd[i];
+        e = capture(c, cs, [mixed, boxed](Ctx& cc) -> cudaError_t {
             cudaError_t r = mixed ? launch_push_mixed(cc) : launch_push(cc);
             if (r == cudaSuccess) r = mixed ? launch_movers_mixed(cc) : launch_movers(cc);
             if (r == cudaSuccess) r = mixed ? launch_inject_mixed(cc) : launch_inject(cc);
             if (r == cudaSuccess) r = mixed ? launch_rebin_mixed(cc) : launch_rebin(cc);
-            if (r == cudaSuccess && !cc.external_E) r = launch_solve_prefix(cc, cc.stream, fd);
+            if (r == cudaSuccess && !cc.external_E) r = launch_solve_prefix(cc, cc.stream, boxed);
             return r;
         }, &sub);
         if (e == cudaSuccess) e = cudaGraphAddChildGraphNode(&pre[i], g, nullptr, 0, sub);
@@ -206,9 +201,8 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             cudaGraph_t sub = nullptr;
             e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
-                cudaError_t e2 = uses_fd(b, c)
-                                     ? launch_pcg_fd_cluster(c, gsz, cs)
-                                     : launch_pcg_cluster(make_item(c), gsz, smem, mixed, cs);
+                cudaError_t e2 = fd[i] ? launch_pcg_fd_cluster(c, gsz, cs)
+                                       : launch_pcg_cluster(make_item(c), gsz, smem, mixed, cs);
                 e = cudaStreamEndCapture(cs, &sub);
                 if (e == cudaSuccess) e = e2;
             }

@@ -1007,9 +1007,12 @@ static FdArgs fd_args(Ctx& c) {
     return a;
 }
 
-// a batched solve: the system of c on one cluster of C CTAs (1..16)
-cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st) {
+// the cluster kernel's launch for the plan d, split for a team of C CTAs (1..16);
+// ok: the device runs it (a split exists and the cluster fits)
+static cudaError_t fd_cluster_config(const Ctx& c, FdPlan& d, int C, cudaLaunchConfig_t& cfg,
+                                     cudaLaunchAttribute& attr, bool& ok) {
     void* kern = (void*)k_pcg_fd_cluster;
+    ok = false;
     int optin = 0;
     cudaFuncAttributes fa;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c.device);
@@ -1019,29 +1022,52 @@ cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st) {
     const int limit = optin - (int)fa.sharedSizeBytes;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    FdArgs a = fd_args(c);
-    a.maxit = c.maxit;
-    a.d.deep = true;   // (a batch's clusters solve in one refinement step, as the Jacobi clusters do)
-    if (!fd_split(a.d, C, (size_t)limit)) return cudaErrorInvalidConfiguration;
-    cudaLaunchConfig_t cfg = {};
+    if (e != cudaSuccess || !fd_split(d, C, (size_t)limit)) return e;
     cfg.gridDim = dim3((unsigned)C);
     cfg.blockDim = dim3(FD_THREADS);
-    cfg.dynamicSmemBytes = fd_smem(a.d);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
+    cfg.dynamicSmemBytes = fd_smem(d);
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)C;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int nclusters = 0;
     e = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
+    ok = e == cudaSuccess && nclusters >= 1;
+    return e;
+}
+
+// The CTAs of a member's cluster (0: none can run it): the smallest power of two
+// that keeps each CTA at or under cta_nodes nodes and whose CTAs take a plane's
+// columns between them (a long x axis has more 16-column tiles than few CTAs hold).
+int fd_cluster_size(const Ctx& c, long long cta_nodes) {
+    for (int C = 1; C <= 16; C *= 2) {
+        if (C < 16 && (c.mesh.nnodes + C - 1) / C > cta_nodes) continue;
+        FdPlan d = c.fd;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr = {};
+        bool ok;
+        if (fd_cluster_config(c, d, C, cfg, attr, ok) != cudaSuccess) cudaGetLastError();
+        else if (ok) return C;
+    }
+    return 0;
+}
+
+// a batched solve: the system of c on one cluster of C CTAs (fd_cluster_size)
+cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st) {
+    FdArgs a = fd_args(c);
+    a.maxit = c.maxit;
+    a.d.deep = true;   // (a batch's clusters solve in one refinement step, as the Jacobi clusters do)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    bool ok;
+    cudaError_t e = fd_cluster_config(c, a.d, C, cfg, attr, ok);
     if (e != cudaSuccess) return e;
-    if (nclusters < 1) return cudaErrorInvalidConfiguration;
+    if (!ok) return cudaErrorInvalidConfiguration;
+    cfg.stream = st;
     void* args[] = {(void*)&a, (void*)&C};
-    return cudaLaunchKernelExC(&cfg, kern, args);
+    return cudaLaunchKernelExC(&cfg, (void*)k_pcg_fd_cluster, args);
 }
 
 cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st) {

@@ -111,15 +111,19 @@ def test_field_solves_between_steps():
 BATCH = [((13, 12, 14), [D] * 6), ((17, 16, 15), [N, D, D, D, N, D]), ((24, 33, 9), [D, D, N, N, D, N]),
          ((31, 18, 47), [D, N, N, D, D, D]), ((48, 46, 49), [D] * 6), ((2, 33, 30), [D, D, N, N, D, N]),
          ((40, 2, 30), [N, D, D, D, N, N]), ((33, 40, 2), [N, N, N, N, D, D]), ((8, 8, 140), [N, D, D, N, D, D])]
+# a long x axis: more 16-column tiles than the CTAs that the node count alone asks for can hold (4; then 1 and 1)
+LONG = [((520, 3, 2), [D] * 6)], [((130, 10, 10), [D] * 6), ((140, 11, 9), [N, D, D, N, D, D])]
 
 
-def test_fast_diagonal_clusters_match_oracle():
+@pytest.mark.parametrize("members,cta_nodes", [(BATCH, 8192), (LONG[0], 8192), (LONG[1], 65536)])
+def test_fast_diagonal_clusters_match_oracle(members, cta_nodes):
     from paper_2011_10214_gb300 import capi
-    pairs = [_pair(n, bc, _sphere(n) if min(n) > 2 else ("none",)) for n, bc in BATCH]
+    pairs = [_pair(n, bc, _sphere(n) if min(n) > 2 else ("none",)) for n, bc in members]
     for k, (gpu, orc) in enumerate(pairs):
         add_species_both(gpu, orc, -1.0, 1.0, 0.01)
         explicit_particles(gpu, orc, 0, 3000, 50 + k, 0.5)
     batch = capi.Batch([gpu for gpu, _ in pairs])
+    batch.set_cta_nodes(cta_nodes)
     for _ in range(2):
         st = batch.step(1)
         for k, (gpu, orc) in enumerate(pairs):
@@ -128,7 +132,7 @@ def test_fast_diagonal_clusters_match_oracle():
             F = gpu.node_charge(0) * (-0.01 / 2.0 ** 32)
             qT = orc.fs.q_tets(-0.01 * gpu.surface_counts(0).astype(np.float64))
             phi, _, _ = orc.fs.solve(F, qT, tol=1e-12, maxit=5000)
-            assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max(), BATCH[k]
+            assert np.abs(gpu.potential() - phi).max() <= TOL_PHI * np.abs(phi).max(), members[k]
     batch.close()
     for gpu, _ in pairs:
         gpu.close()
