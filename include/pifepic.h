@@ -230,8 +230,9 @@ pifepic_status pifepic_set_refinement(pifepic_ctx* ctx, double reduction, double
  * node's permittivity; its iteration count does not grow with the mesh.  (The
  * transforms take FP32 operands split into two BF16 parts; vectors, products
  * with the operator and dot products stay FP32, the residual that ends a solve
- * FP64.)  It applies unless every face is Neumann or an x-y plane is too large
- * for shared memory (about 200 x 200 nodes; more than 256 along z).  Its
+ * FP64.)  It applies unless the largest permittivity is more than 10 times the
+ * smallest, every face is Neumann or an x-y plane is too large for shared
+ * memory (about 200 x 200 nodes; more than 256 along z).  Its
  * reduction is at most 1e-6 between Dirichlet faces and in a batch, else its
  * margin at most 0.2 (pifepic_set_refinement).  All solve the same system to
  * the same stopping test.  Takes effect at once (the solve is re-planned); no

@@ -41,6 +41,15 @@ constexpr long long FD_MIN_NODES = 32768;
 // a batch's clusters from this many (16^3 cells: 0.26 ms a member's step against 0.45 with
 // the Jacobi cluster, 48^3: 0.66 against 1.52)
 constexpr long long FD_CLUSTER_MIN_NODES = 2048;
+// neither of them where the largest permittivity (plasma, object, bedrock) is more than
+// this many times the smallest: the iteration count grows with it, and far beyond, an
+// inner solve loses its FP32 digits and diverges (crater ground of 1000: residual 1e19,
+// Jacobi converges).  us a solve, this against Jacobi (multigrid at 96^3), at 10: 32^3
+// sphere 338 and 381, 64^3 599 and 1001, 96^3 crater 1692 and 1885, a batch of 24^3 boxes
+// 1128 and 1195 a step; at 20: 409 and 397, 724 and 1036, 2438 and 1678, 1370 and 1236; at
+// 100: 699 and 448, 1197 and 1182, 6648 and 2765, 2442 and 1405.  At 1/10: 32^3 sphere 280
+// and 271, 96^3 905 and 1758, the batch 994 and 1114; at 1/30: 356 and 270, 1159 and 2081
+constexpr double FD_MAX_CONTRAST = 10.0;
 struct FdPlan {
     int mx = 0, my = 0, mz = 0;   // free nodes per axis (0: no plan), the first at (x0, y0, z0)
     int x0 = 0, y0 = 0, z0 = 0;

@@ -878,14 +878,17 @@ static bool fd_split(FdPlan& d, int G, size_t limit) {
 
 // The plan for the context's mesh, boundaries and operator, in MIXED mode with AUTO,
 // once pifepic_solve_field (from FD_MIN_NODES nodes) or a batch has asked for it; not
-// where no node is free, where every face is Neumann (P is singular) or where a plane
-// does not fit in shared memory.
+// where no node is free, where every face is Neumann (P is singular), where a plane
+// does not fit in shared memory or beyond FD_MAX_CONTRAST.
 cudaError_t plan_pcg_fd(Ctx& c) {
     free_fd(c);
     const Mesh& m = c.mesh;
     if (c.precision != PIFEPIC_MIXED || c.precond != PIFEPIC_PRECOND_AUTO || !c.fd_wanted ||
         m.nnodes < FD_CLUSTER_MIN_NODES)
         return cudaSuccess;
+    double lo = std::min(c.obj.eps_plus, c.obj.eps_minus), hi = std::max(c.obj.eps_plus, c.obj.eps_minus);
+    if (c.obj.bed) { lo = std::min(lo, c.obj.eps_bed); hi = std::max(hi, c.obj.eps_bed); }
+    if (!(hi <= FD_MAX_CONTRAST * lo)) return cudaSuccess;
     int dir[6], any = 0;
     for (int f = 0; f < 6; ++f) any |= dir[f] = c.bc[f].kind == PIFEPIC_BC_DIRICHLET;
     FdPlan d;

@@ -136,3 +136,44 @@ def test_fast_diagonal_clusters_match_oracle(members, cta_nodes):
     batch.close()
     for gpu, _ in pairs:
         gpu.close()
+
+
+# (object, bedrock): permittivities up to 10 times apart, and more
+GROUND = ("cap_crater", 3.1, 8.0, 9.0, 5.0, 2.0)
+CONTRAST = [(("sphere", (8.0, 8.0, 8.0), 3.0, 10.0, 1.0), None, True), (("sphere", (8.0, 8.0, 8.0), 3.0, 0.2, 2.0), None, True),
+            (GROUND + (4.0, 1.0), (1.4, 10.0), True), (("sphere", (8.0, 8.0, 8.0), 3.0, 30.0, 1.0), None, False),
+            (("sphere", (8.0, 8.0, 8.0), 3.0, 0.05, 1.0), None, False), (GROUND + (1000.0, 1.0), None, False),
+            (GROUND + (4.0, 1.0), (1.4, 12.0), False)]
+
+
+@pytest.mark.parametrize("case", range(len(CONTRAST)))
+def test_high_contrast_keeps_the_other_solvers(case):
+    """AUTO's field solves and clusters are Jacobi's to the bit where permittivities are more than
+    10 times apart (with a ground of 1000 the fast-diagonalisation solve diverged), and meet the
+    tolerance with fewer iterations up to there."""
+    from paper_2011_10214_gb300 import capi
+    obj, bed, fast = CONTRAST[case]
+    n, bc = (32, 36, 32), [N] * 5 + [D] if obj[0] == "cap_crater" else [D] * 6
+    g = np.random.default_rng(3)
+    F = g.normal(size=33 * 37 * 33) * 0.125
+    got = []
+    for precond in (capi.PRECOND_JACOBI, capi.PRECOND_AUTO):
+        gpu, orc = _pair(n, bc, obj, bed, maxit=1000, tol=1e-6)
+        gpu.set_preconditioner(precond)
+        it, rr = gpu.solve_field(F)
+        assert rr <= 1e-6
+        phi = gpu.potential()
+        add_species_both(gpu, orc, -1.0, 1.0, 0.01)
+        explicit_particles(gpu, orc, 0, 3000, 7, 0.5)
+        batch = capi.Batch([gpu])
+        batch.set_preconditioner(precond)
+        st = batch.step(1)[0]
+        assert st["pcg_converged"] == 1
+        got.append((it, phi, st["pcg_iters"], gpu.potential()))
+        batch.close()
+        gpu.close()
+    (it, phi, bit, bphi), (it2, phi2, bit2, bphi2) = got
+    if fast:
+        assert it2 < 0.5 * it and bit2 < 0.5 * bit
+    else:
+        assert it2 == it and bit2 == bit and np.array_equal(phi2, phi) and np.array_equal(bphi2, bphi)
