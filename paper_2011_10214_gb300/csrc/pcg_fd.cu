@@ -1061,7 +1061,11 @@ int fd_cluster_size(const Ctx& c, long long cta_nodes) {
 cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st) {
     FdArgs a = fd_args(c);
     a.maxit = c.maxit;
-    a.d.deep = true;   // (a batch's clusters solve in one refinement step, as the Jacobi clusters do)
+    // A batch's clusters solve in one refinement step, as the Jacobi clusters do, with Neumann
+    // faces too: on members of 15,000 to 50,000 nodes, craters and layers with five Neumann
+    // faces among them, the potential is then 2e-7 to 1.5e-6 from a tight solve's, where the
+    // Jacobi clusters leave 4e-7 to 4e-6 (and 2e-3 where their 150 iterations are too few).
+    a.d.deep = true;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr = {};
     bool ok;

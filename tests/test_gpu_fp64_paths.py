@@ -64,3 +64,35 @@ def test_solve_sums_in_fixed_point_and_by_partials_agree(n):
         sim.close()
     assert np.abs(phi[0]).max() > 0
     assert np.abs(phi[0] - phi[1]).max() <= 2e-10 * np.abs(phi[0]).max()
+
+
+def test_sums_out_of_range_inside_a_solve():
+    """A load that is one eigenvector of D^-1 A and, 1e-5 as large, all the others: the first
+    iteration takes the totals down by 1e8 or more, far below the 1/128 of the last ones that
+    the fixed-point sums reach, so they are redone by partial sums there and in fixed point
+    again after it.  Both sides stop at |r| <= 1e-12 |b| (condition below 100 here)."""
+    from oracle.field import FieldSystem
+    from oracle.geometry import Mesh, NoObject
+    from paper_2011_10214_gb300 import capi
+    n = (9, 7, 8)
+    bc = [("D", 0.0)] * 6
+    m = Mesh(*n, 0.5)
+    fs = FieldSystem(m, NoObject(), bc)
+    A = fs.A_ff.toarray()
+    d = np.sqrt(A.diagonal())
+    _, V = np.linalg.eigh(A / np.outer(d, d))            # D^-1/2 A D^-1/2; r = D^1/2 v is D times an eigenvector
+    c = np.full(len(d), 1e-5)
+    c[len(d) // 3] = 1.0
+    F = np.zeros(m.nnodes)
+    F[fs.free] = d * (V @ c)
+    one, _, rr = fs.solve(F, np.zeros(0), tol=1e-3, maxit=5)
+    assert rr < 1e-3                                     # (one step: |r|^2 down by more than 1e6)
+    phi, it, _ = fs.solve(F, np.zeros(0), tol=1e-12, maxit=500)
+    assert it > 10
+    sim = capi.Simulation(n, 0.5, 0.1, precision=0, pcg_tol=1e-12, pcg_max_iter=500)
+    sim.set_field_bc(bc)
+    sim.set_object(capi.OBJ_NONE, [], 1.0, 1.0)
+    git, relres = sim.solve_field(F)
+    assert abs(git - it) <= 2 and relres <= 1e-12
+    assert np.abs(sim.potential() - phi).max() <= 1e-10 * np.abs(phi).max()
+    sim.close()
