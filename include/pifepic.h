@@ -426,7 +426,9 @@ pifepic_status pifepic_batch_set_cta_nodes(pifepic_batch* batch, int cta_nodes);
  * clusters of the member's whole working set in shared memory; AUTO (the
  * default) solves the members that the fast-diagonalisation preconditioner
  * applies to (pifepic_set_preconditioner; here from 2048 nodes) by that PCG on
- * one cluster each, the others by Jacobi.
+ * one cluster each, or on the whole device beyond the register-resident solver,
+ * the others by Jacobi (by their own solver where they are too large for a
+ * cluster).
  * FP64 batches always use Jacobi.  The graph is rebuilt on the next step.
  * EINVAL for an unknown kind. */
 pifepic_status pifepic_batch_set_preconditioner(pifepic_batch* batch, int kind);

@@ -28,6 +28,7 @@ cudaError_t build_pcg_graph(Ctx& c);                                            
 cudaError_t launch_pcg_mg_cluster(Ctx& c, int C, cudaStream_t st);                 // pcg_mg.cu
 int fd_cluster_size(const Ctx& c, long long cta_nodes);                             // pcg_fd.cu
 cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st);
+cudaError_t launch_pcg_fd(Ctx& c, cudaStream_t st);
 cudaError_t plan_pcg_fd(Ctx& c);
 size_t cluster_smem_for(long long N, long long H, int C, bool mixed);
 cudaError_t launch_pcg_cluster(const BatchItem& item, int C, size_t smem, bool mixed, cudaStream_t st);
@@ -123,8 +124,8 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
     // the solve of each instance: csize = its Jacobi cluster size (0: too large
     // for a cluster, the single-instance persistent solver); members solved by
     // the multigrid cluster kernel (MIXED, with a hierarchy) get csize -2 and
-    // their cluster size in mg_c, those by the fast-diagonalisation one its
-    // cluster size in csize and a mark in fd
+    // their cluster size in mg_c, those by fast diagonalisation a mark in fd and
+    // its cluster size in csize (or 0, the whole device)
     std::vector<int> csize(n, -1), mg_c(n, 0);
     std::vector<char> fd(n, 0);
     std::vector<int> mg_members;
@@ -146,14 +147,17 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
             continue;
         }
         csize[i] = cluster_size_for(c.mesh.nnodes, node_halo(c.mesh), mixed, b->cta_nodes);
-        if (mixed && csize[i] > 0 && b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx == 0 && !c.fd_wanted) {
-            // the plan on first use (no memory for it: Jacobi)
+        // (a member too large for a cluster that fits the register-resident solver keeps Jacobi)
+        if (!mixed || b->precond != PIFEPIC_PRECOND_AUTO || (csize[i] == 0 && c.pcg_npt > 0)) continue;
+        if (c.fd.mx == 0 && !c.fd_wanted) {
+            // the plan on first use (no memory for it: the other solvers)
             c.fd_wanted = true;
             if (plan_pcg_fd(c) != cudaSuccess) cudaGetLastError();
         }
-        if (csize[i] > 0 && b->precond == PIFEPIC_PRECOND_AUTO && c.fd.mx > 0) {
-            const int C = fd_cluster_size(c, b->cta_nodes / FD_CTA_SHARE);
-            if (C > 0) { csize[i] = C; fd[i] = 1; }
+        if (c.fd.mx > 0) {
+            const int C = csize[i] > 0 ? fd_cluster_size(c, b->cta_nodes / FD_CTA_SHARE) : 0;
+            fd[i] = C > 0 || csize[i] == 0;
+            if (C > 0) csize[i] = C;
         }
     }
     b->plan_gen.resize(n);
@@ -231,7 +235,10 @@ static cudaError_t build_batch_graph(pifepic_batch* b) {
         if (e != cudaSuccess) break;
         Ctx& c = b->ctx[i]->c;
         cudaGraph_t sub = nullptr;
-        e = capture(c, cs, [](Ctx& cc) -> cudaError_t { return launch_pcg_coop(cc, cc.stream); }, &sub);
+        const bool boxed = fd[i];
+        e = capture(c, cs, [boxed](Ctx& cc) -> cudaError_t {
+            return boxed ? launch_pcg_fd(cc, cc.stream) : launch_pcg_coop(cc, cc.stream);
+        }, &sub);
         cudaGraphNode_t deps[2] = {pre[i], last_big};
         if (e == cudaSuccess) e = cudaGraphAddChildGraphNode(&solve_of[i], g, deps, last_big ? 2 : 1, sub);
         if (sub) cudaGraphDestroy(sub);

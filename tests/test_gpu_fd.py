@@ -206,3 +206,26 @@ def test_default_tolerance_leaves_no_more_than_jacobi():
         assert rr <= 1e-6 and np.linalg.norm(gpu.potential() - phi) <= 2e-5 * np.linalg.norm(phi), n
         batch.close()
         gpu.close()
+
+
+def test_batch_member_beyond_the_register_solver():
+    """673,000 nodes: too many for a cluster, solved by fast diagonalisation on the whole device
+    in an AUTO batch and by the member's own multigrid in a JACOBI one.  Both stop at 1e-11 on
+    the same charges; the condition is some 1e3."""
+    from paper_2011_10214_gb300 import capi
+    from paper_2011_10214_gb300 import workloads as wl
+    cfg = dict(wl.sphere_config(16, 2.0, 1, 1), n=(88, 88, 84))
+    got = []
+    for precond in (capi.PRECOND_AUTO, capi.PRECOND_JACOBI):
+        sim = capi.from_config(cfg, precision=capi.MIXED, pcg_tol=1e-11, pcg_max_iter=500)
+        sim.solve()
+        batch = capi.Batch([sim])
+        batch.set_preconditioner(precond)
+        st = batch.step(1)[0]
+        assert st["pcg_converged"] == 1 and st["pcg_relres"] <= 1e-11
+        got.append((sim.node_charge(0), sim.potential(), st["pcg_iters"]))
+        batch.close()
+        sim.close()
+    (W, phi, it), (W2, phi2, it2) = got
+    assert np.array_equal(W, W2) and it != it2
+    assert np.abs(phi - phi2).max() <= 1e-8 * np.abs(phi2).max()
