@@ -98,7 +98,6 @@ struct FdArgs {
     double* phi;                  // potential out (nodes)
     FdPlan d;
     int npatch;
-    // stopping test and caps of a batched solve; of a context's own (maxit 0) the PCG state holds them
     double tol2, inner_red2, margin2;
     int maxit;
     double* val;
@@ -627,8 +626,7 @@ static __device__ void fd_pcg(const FdArgs& a, Team& team, uint2* sm) {
     const Mesh& m = a.f.m;
     const int TT = (int)team.size(), t0 = (int)team.t0();
     const FdShare h = fd_share(d, team, sm);
-    const bool own = a.maxit == 0;
-    const double tol2 = own ? a.S->tol2 : a.tol2, mar2 = own ? a.S->margin2 : a.margin2;
+    const double tol2 = a.tol2;
     // An inner solve that reduces the residual 1e-6-fold meets the tolerance after one
     // refinement step, but leaves the FP32 rounding of its whole correction in the
     // smoothest modes.  Between Dirichlet faces that is 5e-7 of the potential (64^3
@@ -636,10 +634,9 @@ static __device__ void fd_pcg(const FdArgs& a, Team& team, uint2* sm) {
     // are far softer (7e-4 on the 160 x 160 x 80 crater), so there the context's
     // reduction splits the solve into two refinement steps and the second corrects the
     // first's rounding; a margin of 0.2 at most (one iteration more) leaves 2e-6 there.
-    const double red2 = own ? a.S->inner_red2 : a.inner_red2;
-    const double inner_red2 = d.deep ? fmin(red2, FD_INNER_RED * FD_INNER_RED) : red2;
-    const double margin2 = d.deep ? mar2 : fmin(mar2, FD_MARGIN * FD_MARGIN);
-    const int maxit = own ? a.S->maxit : a.maxit;
+    const double inner_red2 = d.deep ? fmin(a.inner_red2, FD_INNER_RED * FD_INNER_RED) : a.inner_red2;
+    const double margin2 = d.deep ? a.margin2 : fmin(a.margin2, FD_MARGIN * FD_MARGIN);
+    const int maxit = a.maxit;
     int it = 0, outer = 0;
     double bb = 0.0, rr = 0.0;
     bool conv = false, alive = true;
@@ -998,7 +995,7 @@ static FdArgs fd_args(Ctx& c) {
     a.tol2 = c.tol * c.tol;
     a.inner_red2 = c.inner_red * c.inner_red;
     a.margin2 = c.inner_margin * c.inner_margin;
-    a.maxit = 0;
+    a.maxit = c.maxit;
     a.val = c.coop_partial;
     a.arrivals = c.bar64 + BAR64_FD;
     a.fx = c.bar64 + BAR64_FD + FX_LINE;
@@ -1060,7 +1057,6 @@ int fd_cluster_size(const Ctx& c, long long cta_nodes) {
 // a batched solve: the system of c on one cluster of C CTAs (fd_cluster_size)
 cudaError_t launch_pcg_fd_cluster(Ctx& c, int C, cudaStream_t st) {
     FdArgs a = fd_args(c);
-    a.maxit = c.maxit;
     // A batch's clusters solve in one refinement step, as the Jacobi clusters do, with Neumann
     // faces too: on members of 15,000 to 50,000 nodes, craters and layers with five Neumann
     // faces among them, the potential is then 2e-7 to 1.5e-6 from a tight solve's, where the

@@ -229,3 +229,17 @@ def test_batch_member_beyond_the_register_solver():
     (W, phi, it), (W2, phi2, it2) = got
     assert np.array_equal(W, W2) and it != it2
     assert np.abs(phi - phi2).max() <= 1e-8 * np.abs(phi2).max()
+
+
+def test_batch_member_that_never_solved_by_itself():
+    """Its tolerance and cap travel with the batch's launches; on the whole device they were read
+    from the state that only a solve of its own sends, and the solve did not iterate."""
+    from paper_2011_10214_gb300 import capi
+    from paper_2011_10214_gb300 import workloads as wl
+    for n in ((20, 20, 20), (88, 88, 84)):
+        sim = capi.from_config(dict(wl.sphere_config(16, 2.0, 1, 1), n=n), precision=capi.MIXED)
+        batch = capi.Batch([sim])
+        st = batch.step(1)[0]
+        assert st["pcg_converged"] == 1 and st["pcg_iters"] > 0 and st["pcg_relres"] <= 1e-6, n
+        batch.close()
+        sim.close()
