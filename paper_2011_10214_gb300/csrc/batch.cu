@@ -2,9 +2,9 @@
 // launch per step.  Each instance's particle phases (push, movers, injection,
 // rebin) and right-hand side are independent branches of the graph, so small
 // instances overlap on the device; the field solves run on thread-block
-// clusters, one cluster per instance (pcg_cluster.cu), with a one-CTA-per-
-// instance kernel for instances too large for a cluster; the node fields
-// follow as branches again.  The paper runs one problem per job (Sec. 3,
+// clusters, one cluster per instance (pcg_fd.cu, pcg_cluster.cu, pcg_mg.cu), on
+// the whole device, one after another, for instances too large for a cluster;
+// the node fields follow as branches again.  The paper runs one problem per job (Sec. 3,
 // Sec. 5); batching and serving many charging problems is this build's addition
 // on top of the same per-instance method.
 #include <math.h>
@@ -94,7 +94,7 @@ struct pifepic_batch {
     std::vector<pifepic_ctx*> ctx;
     cudaStream_t stream = nullptr;
     int cta_nodes = 8192;
-    int precond = PIFEPIC_PRECOND_AUTO;   // MIXED members: MULTIGRID = multigrid clusters, else Jacobi clusters
+    int precond = PIFEPIC_PRECOND_AUTO;   // MIXED members (pifepic_batch_set_preconditioner)
     bool dirty = true;
     std::vector<unsigned long long> plan_gen;   // the members' Ctx::plan_gen when the graph was built
     std::vector<long long> kernels;   // kernels per step of each instance (its share of the batch graph)

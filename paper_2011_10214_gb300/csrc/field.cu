@@ -1,5 +1,6 @@
-// IFE field solve on the GPU: right-hand side with the flux-jump term, Jacobi
-// PCG with a matrix-free operator plus 19-slot patch rows, node field.
+// IFE field solve on the GPU: right-hand side with the flux-jump term, the solve
+// graph around the persistent PCG kernels (pcg_coop.cu, pcg_mg.cu, pcg_fd.cu),
+// node field, and the statistics of a call.
 //
 // Sec. 2.1 (Eqs. 2.1-2.5): weak form a(phi, v) = (rho, v) - int_Gamma q v; the
 // non-homogeneous IFE solution is phi_h = u_h + phi_J (phi_J the element-wise
@@ -7,13 +8,11 @@
 // psi_i), i.e. F_i + sum_T q_T c_{T,i} (c the unit-jump load of interface tet
 // T).  Sec. 2.5: the matrix solve is a PCG iteration stopped on the relative
 // residual (Sec. 3.2, Sec. 4, Sec. 5.2.2 give tolerance 1e-6 and caps 60/150).
-// Preconditioner (unstated in the paper): Jacobi.
+// Preconditioners (unstated in the paper): pcg_coop.cu, pcg_mg.cu and pcg_fd.cu.
 //
-// The whole solve is one CUDA graph: q_T, RHS, initial residual, then a
-// conditional WHILE node whose body is one PCG iteration (spmv + p.q, update +
-// r.r + r.z, direction update).  The iteration count and convergence test live
-// on the device; no host round trip.  Reductions are deterministic: per-block
-// partials, summed in a fixed order by the last block to finish.
+// The whole solve of a step is one CUDA graph: q_T, RHS and start vector, one
+// persistent PCG kernel, node field.  The iteration count and convergence test
+// live on the device; no host round trip.
 #include <math.h>
 #include <stdio.h>
 #include <atomic>
@@ -682,8 +681,8 @@ cudaError_t set_field_tables(const TetTables& t) {
 // loop whose device memory is handed out by a pool it does not own (a
 // cudaMalloc there can fail or stall the whole process on a device
 // synchronisation), or an embedding that forbids allocation after start-up.
-// pifepic_solve_field allocates a staging buffer and builds a CUDA graph on
-// every call, so those callers need this variant.  It reuses the context's
+// pifepic_solve_field allocates a staging buffer on every call and its solver's
+// plan on the first, so those callers need this variant.  It reuses the context's
 // operator (read only), takes the load F, the flux jumps q (NULL: none) and
 // the output phi as caller-owned device arrays, and keeps every work vector of
 // the PCG in one file-scope device array of fixed size, found once per device

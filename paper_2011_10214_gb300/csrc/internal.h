@@ -430,13 +430,11 @@ cudaError_t launch_field_lift(Ctx& c);
 cudaError_t build_pcg_graph(Ctx& c);                   // field.cu
 void plan_pcg(Ctx& c);                                 // pcg_coop.cu
 cudaError_t launch_pcg(Ctx& c);
-// diag: also the surface charge and mean surface potential (a few kernels)
 // statistics of a call over n contexts: mark_stats queues the reading of the
 // counters before it, queue_stats the gathering after it, into each context's
 // stat_host[1] and [0]; both are there once st has been waited for
 cudaError_t mark_stats(Ctx* const* c, int n, cudaStream_t st);
 cudaError_t queue_stats(Ctx* const* c, int n, cudaStream_t st);
-cudaError_t launch_qtets(Ctx& c);
 
 Launch make_launch(Ctx& c);
 cudaError_t launch_load_maxwellian(Ctx& c, int s, int ppc, double vth, const double drift[3],

@@ -463,8 +463,8 @@ static __device__ __forceinline__ void fd_deal(const Team& team, int nw, int np,
 //   eps (cx (c0 cy cz h z - h/6 (cz Sy + cy Sz) - h/12 Dyz) - h/6 cy cz Sx
 //        - h/12 (cz Dxy + cy Dxz)),
 // c0 = 3/4 and the diagonals on even nodes, c0 = 1/2 and none on odd ones.  The patch
-// rows are a list of their own, 32 to a warp, after the regular ones: met among these
-// they would set the pace of every block that has some.  z goes through L1: the team's
+// rows are a list of their own, 32 to a warp, before the regular ones (fd_deal): met among
+// these they would set the pace of every warp that has some.  z goes through L1: the team's
 // last barrier ordered the writers before these reads.
 template <class Team>
 static __device__ void fd_matvec(const FdArgs& a, const Team& team, int cur, float (&v)[2]) {
