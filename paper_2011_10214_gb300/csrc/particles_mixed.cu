@@ -22,20 +22,34 @@ __global__ void k_bin_scan(int nb, const int* cap, long long* start, long long* 
 __global__ void k_clamp_counts(Launch L, long long* step);
 cudaError_t launch_push_prep(Ctx& c);
 
+// Which product of a b + c d is rounded before the fused sum: ROUND 1 the first, 2 the
+// second, 0 either, as the compiler likes.  The bins' push pins it, 2 at a move's start
+// and 1 at its end (its order when one pass did all): it takes the level set of a particle
+// in two places, and left to the compiler 1 hit in 2 million (sphere; 1 in 700,000 on a
+// plane, 1 in 12 million on a cap crater) within rounding of the surface or of a cell's
+// face was decided differently than before the leavers had a pass of their own.
+template <int ROUND>
+PF_D float sum2(float a, float b, float c, float d) {
+    return ROUND == 1 ? fmaf(c, d, a * b) : ROUND == 2 ? fmaf(a, b, c * d) : a * b + c * d;
+}
+
+template <int ROUND = 0>
 PF_D float level_set_f(const ObjF& o, float x, float y, float z) {
     if (o.kind == 1) {
         float dx = x - o.a0, dy = y - o.a1, dz = z - o.a2;
+        if (ROUND) return fmaf(dz, dz, sum2<ROUND>(dx, dx, dy, dy)) - o.a3;
         return (dx * dx + dy * dy + dz * dz) - o.a3;
     } else if (o.kind == 2) {
         float dx = x - o.a1, dy = y - o.a2;
-        float r2 = dx * dx + dy * dy;
+        float r2 = sum2<ROUND>(dx, dx, dy, dy);
         float zs = (r2 < o.a3) ? o.a5 - sqrtf(o.a4 - r2) : o.a0;
         return z - zs;
     } else if (o.kind == 3) {
+        if (ROUND) return fmaf(o.a2, z, sum2<ROUND>(o.a0, x, o.a1, y)) - o.a3;
         return o.a0 * x + o.a1 * y + o.a2 * z - o.a3;
     } else if (o.kind == 4) {   // rim crater, parameters as in level_set
         const float dx = x - o.a0, dy = y - o.a1;
-        const float r = sqrtf(dx * dx + dy * dy);
+        const float r = sqrtf(sum2<ROUND>(dx, dx, dy, dy));
         float zs;
         if (r <= o.a2) {
             zs = o.a5;
@@ -159,8 +173,9 @@ PF_D void reflect_axis_pf(float& x, float& v, int n, int lo, int hi) {
     }
 }
 
+template <bool PIN = false>
 PF_D int hit_cell_f(const Launch& L, const ObjF& of, float xo, float yo, float zo, float xn, float yn, float zn) {
-    float Lo = level_set_f(of, xo, yo, zo), Ln = level_set_f(of, xn, yn, zn);
+    float Lo = level_set_f<PIN ? 2 : 0>(of, xo, yo, zo), Ln = level_set_f<PIN ? 1 : 0>(of, xn, yn, zn);
     float t = Lo / (Lo - Ln);
     float xc = xo + t * (xn - xo), yc = yo + t * (yn - yo), zc = zo + t * (zn - zo);
     // the crossing point's cell on the IFE mesh (refine times finer; exact scaling)
@@ -171,7 +186,7 @@ PF_D int hit_cell_f(const Launch& L, const ObjF& of, float xo, float yo, float z
     return L.cell_acc[cell_id(L.fmesh, ci, cj, ck)];
 }
 
-template <class EA>
+template <bool PIN = false, class EA>
 PF_D int push_one(const Launch& L, const ObjF& of, float kf, float dthf, int refl, PF32& p, const EA& ea, int& acc) {
     WF w = weights_f(p.fx, p.fy, p.fz);
     float ex, ey, ez;
@@ -183,8 +198,8 @@ PF_D int push_one(const Launch& L, const ObjF& of, float kf, float dthf, int ref
     if (refl) reflect_cell(L.mesh, refl, p);
     if (p.i < 0 || p.i >= L.mesh.nx || p.j < 0 || p.j >= L.mesh.ny || p.k < 0 || p.k >= L.mesh.nz) return ABSORBED;
     float xn = (float)p.i + p.fx, yn = (float)p.j + p.fy, zn = (float)p.k + p.fz;
-    if (level_set_f(of, xn, yn, zn) < 0.0f) {
-        acc = hit_cell_f(L, of, xo, yo, zo, xn, yn, zn);
+    if (level_set_f<PIN ? 1 : 0>(of, xn, yn, zn) < 0.0f) {
+        acc = hit_cell_f<PIN>(L, of, xo, yo, zo, xn, yn, zn);
         return COLLECTED;
     }
     return ALIVE;
@@ -379,7 +394,7 @@ static __device__ __noinline__ void push_leavers(const Launch& L, const SpeciesD
                 return second ? make_float4(p.y, p.w, q.y, 0.0f) : make_float4(p.x, p.z, q.x, 0.0f);
             }
         };
-        code = push_one(L, of, (float)S.k, dthf, S.reflect, p, Tile{P, Q, x0, y0, z0}, acc);
+        code = push_one<true>(L, of, (float)S.k, dthf, S.reflect, p, Tile{P, Q, x0, y0, z0}, acc);
         if (code == COLLECTED && acc >= 0) atomicAdd(&S.surf[acc], 1ull);
     }
     count_event32(&sctr[C_ABSORBED], code == ABSORBED);
@@ -536,7 +551,7 @@ __global__ void __launch_bounds__(32 * NW, RF == 2 ? 3 : 32 / NW) k_push_bins_m(
         bool stay = live & ((unsigned)ri < (unsigned)lx) & ((unsigned)rj < (unsigned)ly) & ((unsigned)rk < (unsigned)lz);
         if (!clear)
             stay = stay &&
-                   !(level_set_f(of, (float)(ri + x0) + fx, (float)(rj + y0) + fy, (float)(rk + z0) + fz) < 0.0f);
+                   !(level_set_f<1>(of, (float)(ri + x0) + fx, (float)(rj + y0) + fy, (float)(rk + z0) + fz) < 0.0f);
         const unsigned bal = __ballot_sync(0xffffffffu, stay);
         // refill the stage slot: the bulk copy is not ordered after the reads of the slot by
         // itself, but the vote above has waited for what every lane made of its seven words
